@@ -3,6 +3,7 @@
 // schedule of Algorithm 1.
 #include <algorithm>
 #include <climits>
+#include <cmath>
 #include <cstring>
 
 #include "edp.h"
@@ -244,6 +245,16 @@ int check_range(int W, int H, const Geometry &g, const edp_params *p) {
     return EDP_OK;
 }
 
+// Spaces the whole-line (lean) form of the multi-axis kernel serves.
+bool lean_space(const Geometry &g) {
+    bool short_lines = g.R >= 2, all65 = g.R >= 2;
+    for (int r = 0; r < g.R; ++r) {
+        short_lines = short_lines && (g.Qr[r] == 9 || g.Qr[r] == 17 || g.Qr[r] == 33);
+        all65 = all65 && g.Qr[r] == 65;
+    }
+    return short_lines || all65;
+}
+
 // Multi-axis kernel shape: warps per row (team), per-axis lane groups.
 // Cost model of one column step: every round of an axis runs the two
 // in-lane sweeps over E labels; lane groups add the carry exchange.
@@ -293,7 +304,8 @@ bool team_shape(const Geometry &g, int T, int gpar, TeamShape *S) {
 struct SolvePlan {
     bool r1;          // warp-per-row body (one label axis, Q <= 256)
     bool line;        // two-axis line kernel (one label line per lane)
-    bool split;       // its form with each line split over two lanes
+    bool split;       // the split line kernel (two or three axes)
+    int build;        // its build
     int Q0, Q1;       // its label-space shape
     int nbands;
     int threads;
@@ -304,6 +316,148 @@ struct SolvePlan {
     PassR1Args o;
     TeamArgs ta;
 };
+
+// Fields of the multi-axis argument block shared by its kernels.
+void fill_team(TeamArgs &a, const int32_t *C, int *const M[4], int32_t *labels, unsigned char *ws,
+               const SolveLayout &L, int W, int H, const Geometry &g, const edp_params *p) {
+    a.C = C;
+    for (int k = 0; k < 4; ++k) a.M[k] = M[k];
+    a.labels = labels;
+    a.ll = reinterpret_cast<int2 *>(ws + L.ll);
+    a.status = reinterpret_cast<int *>(ws);
+    a.W = W;
+    a.H = H;
+    a.Q = g.Q;
+    a.Qm = L.Qm;
+    a.R = g.R;
+    a.lam = p->lambda;
+    a.capv = (int)cap_value(p);
+    a.mode = p->prior_mode;
+    a.l1 = p->l1;
+    a.g = p->g;
+    a.spin_limit = g_spin_limit;
+}
+
+// Shape of the split line kernel (pass_line2.cuh): per axis the segments per
+// line, the compute warps T of a row and the rows NT of a block, by estimated
+// time in SM cycles (a warp's instructions of a phase take kDep times as long
+// when few warps share the scheduler, and the schedulers issue kIpc a cycle).
+struct Line2Shape {
+    int build, T, NT, nst, occ;
+    SegAxis seg[3];
+    int E[3];
+    double cost;
+};
+// The cut of the axes by build b; false if its lines do not fit.
+bool line2_cut(const Geometry &g, const edp_params *p, int b, Line2Shape *S) {
+    const Line2Build &B = pass_line2_build(b);
+    if ((B.S[2] > 0 ? 3 : 2) != g.R) return false;
+    for (int r = 0; r < g.R; ++r) {
+        const int L = g.Qr[r], s = B.S[r], e = (L + s - 1) / s;
+        if (L < s || e > B.E[r] || (B.exact && e != B.E[r])) return false;
+        S->E[r] = e;
+        S->seg[r].S = s;
+        S->seg[r].lpw = 32 / s;
+        S->seg[r].nf = L - s * (e - 1);
+        S->seg[r].kc = std::min(s - 1, (p->g - 1 + L / s - 1) / (L / s));
+    }
+    S->build = b;
+    return true;
+}
+bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, int sms, int rows, int warps,
+                 Line2Shape *best) {
+    constexpr double kDep = 4.5, kIpc = 2.5, kFixed = 400.0, kHop = 2600.0;
+    bool have = false;
+    for (int b = 0; b < pass_line2_builds(); ++b) {
+        const Line2Build &B = pass_line2_build(b);
+        Line2Shape S;
+        memset(&S, 0, sizeof S);
+        if (!line2_cut(g, p, b, &S)) continue;
+        for (int T = 1; T <= pass_line2_max_warps(); ++T) {
+            if (warps > 0 && T != warps) continue;
+            S.T = T;
+            double ins[3] = {0, 0, 0}, busy[3] = {0, 0, 0};  // instructions of a warp, warps at work, per phase
+            int most = 1;
+            for (int r = 0; r < g.R; ++r) {
+                const int lpw = S.seg[r].lpw, n = (r == 0 ? 1 : 2) * ((g.Q / g.Qr[r] + lpw - 1) / lpw);
+                const int rounds = (n + T - 1) / T;
+                most = std::max(most, n);
+                ins[r] = rounds * ((r == 0 ? 24.0 : 11.0) * B.E[r] * (B.exact ? 1.0 : 1.3) + 45.0);
+                busy[r] = (double)n / rounds;
+            }
+            if (warps <= 0 && T > most) break;
+            for (int NT = 1; NT <= 8; ++NT) {
+                if (rows > 0 && NT != std::min(rows, H)) continue;
+                if (NT > H || pass_line2_threads(NT, T) > B.threads) break;
+                S.NT = NT;
+                S.nst = 4;
+                while (S.nst > 2 && pass_line2_smem(NT, Qm, S.nst) > (size_t)kMaxSmem) --S.nst;
+                const size_t smem = pass_line2_smem(NT, Qm, S.nst);
+                if (smem > (size_t)kMaxSmem) break;
+                S.occ = std::max(1, std::min(B.threads / pass_line2_threads(NT, T),
+                                             (int)(kMaxSmem / (smem + 1024))));
+                const int nb = (H + NT - 1) / NT;
+                const bool resident = nb <= S.occ * sms;
+                const int per_sm = resident ? (nb + sms - 1) / sms : S.occ;
+                double step = kFixed;
+                for (int r = 0; r < g.R; ++r) step += std::max(kDep * ins[r], per_sm * NT * busy[r] * ins[r] / kIpc);
+                const double run = std::min(H, S.occ * sms * NT);
+                const double fill = run * (step + kHop / NT);
+                S.cost = resident ? 2.0 * W * step + fill : std::ceil(2.0 * nb / (S.occ * sms)) * W * step + fill;
+                if (!have || S.cost < best->cost) {
+                    *best = S;
+                    have = true;
+                }
+            }
+        }
+    }
+    return have;
+}
+bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry &g, const edp_params *p,
+                int32_t *labels, unsigned char *ws, int sms, SolvePlan *P) {
+    // lambda 255 (the heaviest per-edge multiplier) within the sweeps' range;
+    // 16-byte bulk copies of C
+    if (g.R < 2 || (long long)p->lambda * 255 > pass_line2_max_lambda() ||
+        (reinterpret_cast<uintptr_t>(C) & 15))
+        return false;
+    const SolveLayout &L = P->L;
+    Line2Shape S;
+    // the tuning hooks' shape if there is one, else the planner's own
+    if (!line2_shape(g, p, W, H, L.Qm, sms, g_tune_rb, g_tune_t, &S) && !line2_shape(g, p, W, H, L.Qm, sms, 0, 0, &S))
+        return false;
+    P->line = P->split = true;
+    P->Q0 = g.Qr[0];
+    P->Q1 = g.Qr[1];
+    TeamArgs &a = P->ta;
+    fill_team(a, C, M, labels, ws, L, W, H, g, p);
+    int stride = 1;
+    for (int r = 0; r < 3; ++r) {
+        const int n = r < g.R ? g.Qr[r] : 1;
+        a.ax[r] = TeamAxis{n, S.seg[r].S, S.E[r], g.Q / n, stride, S.seg[r].kc, 1};
+        a.seg[r] = S.seg[r];
+        stride *= n;
+    }
+    a.T = S.T;
+    a.NT = S.NT;
+    a.nbuf = S.nst;
+    a.nbands = (H + S.NT - 1) / S.NT;
+    // hand-off ring (plain values, 4 bytes a label; the consumer counts a
+    // column nst columns late): 8 columns of slack when every band is resident,
+    // otherwise the depth that lets the first resident band finish its row
+    P->nbands = a.nbands;
+    P->build = S.build;
+    P->threads = pass_line2_threads(S.NT, S.T);
+    P->smem = pass_line2_smem(S.NT, L.Qm, S.nst);
+    const int occ = edp_pass_line2_occupancy(P->build, P->threads, P->smem);
+    const int need = S.nst + (a.nbands <= occ * sms ? 8 : team_ring(W, std::max(1, occ * sms)));
+    a.ring = std::min(need, 2 * team_ring(2 * W, kResidentMin));
+    if (occ < 1 || a.ring < need) {  // (cannot happen with the SMs the workspace was sized for)
+        memset(&P->ta, 0, sizeof P->ta);
+        P->line = P->split = false;
+        return false;
+    }
+    return true;
+}
 
 int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_params *p, int32_t *labels,
                unsigned char *ws, SolvePlan *P, int fixed_threads = 0) {
@@ -357,11 +511,19 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
         P->em = a.EMt;
         return EDP_OK;
     }
-    // two label axes with a build of the line kernel (one label line per
-    // lane): single-problem solves of the linear prior
-    // (measured: faster than the whole-line multi-axis form where lines hold
-    // 65 labels, whose rows the multi-axis kernel cannot all keep resident;
-    // slower at 33 x 33)
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    // split line kernel: linear prior, single-problem solves (g_line_mode:
+    // 0 every space it serves, 2 65 x 65 labels only, 1 never)
+    const bool is65 = g.R == 2 && g.Qr[0] == 65 && g.Qr[1] == 65;
+    if (!fixed_threads && !g_generic_team && g_line_split && g_line_mode != 1 && p->l1 == 1 &&
+        (is65 || (g_line_mode == 0 && !g_force_general)) && plan_line2(C, M, W, H, g, p, labels, ws, sms, P))
+        return EDP_OK;
+    // two label axes with a build of the one-lane line kernel: single-problem
+    // solves on request, and above the split kernel's lambda bound where lines
+    // hold 65 labels (the multi-axis kernel cannot keep all their rows resident)
     // The quadratic prior: the line kernel serves the shapes it has a build
     // for (no other form serves them with l1 = 2).
     const bool line_pick = g_line_mode == 2 ||
@@ -370,17 +532,7 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
         P->line = true;
         P->Q0 = g.Qr[0];
         P->Q1 = g.Qr[1];
-        // lines split over lane pairs where built; the completions of the
-        // split sweeps add up to 33 lambda, bounded here for the heaviest
-        // per-edge multiplier (255)
-        P->split = g_line_split && pass_line_split_built(P->Q0, P->Q1, p->l1) &&
-                   (long long)p->lambda * 255 <= pass_line_split_max_lambda();
-        const bool split = P->split;
-        const int TW = pass_line_warps(P->Q0, P->Q1, split);
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        sms = std::max(1, sms);
+        const int TW = pass_line_warps(P->Q0, P->Q1);
         // rows per block: every row band resident, the fewest rows on the
         // busiest SM (blocks are spread evenly), then the most rows per block
         // (fewer hand-offs between blocks); one row per block when no shape
@@ -392,9 +544,9 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
             int best = INT_MAX;
             for (int nt = 1; nt <= 4; ++nt) {
                 const int nb = (H + nt - 1) / nt;
-                const size_t sm = pass_line_smem(nt, P->Q0, P->Q1, split);
+                const size_t sm = pass_line_smem(nt, P->Q0, P->Q1);
                 if (sm > (size_t)kMaxSmem) break;
-                const int occ = edp_pass_line_occupancy(P->Q0, P->Q1, p->l1, split, 32 * TW * nt, sm);
+                const int occ = edp_pass_line_occupancy(P->Q0, P->Q1, p->l1, 32 * TW * nt, sm);
                 if (occ < 1 || nb > occ * sms) continue;
                 const int load = nt * ((nb + sms - 1) / sms);
                 if (load <= best) {
@@ -404,24 +556,10 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
             }
         }
         NT = std::max(1, std::min(NT, H));
-        P->smem = pass_line_smem(NT, P->Q0, P->Q1, split);
+        P->smem = pass_line_smem(NT, P->Q0, P->Q1);
         if (P->smem > (size_t)kMaxSmem) return EDP_ERR_UNSUPPORTED;
         TeamArgs &a = P->ta;
-        a.C = C;
-        for (int k = 0; k < 4; ++k) a.M[k] = M[k];
-        a.labels = labels;
-        a.ll = reinterpret_cast<int2 *>(ws + L.ll);
-        a.status = reinterpret_cast<int *>(ws);
-        a.W = W;
-        a.H = H;
-        a.Q = g.Q;
-        a.Qm = L.Qm;
-        a.R = g.R;
-        a.lam = p->lambda;
-        a.capv = (int)cap_value(p);
-        a.mode = p->prior_mode;
-        a.l1 = p->l1;
-        a.g = p->g;
+        fill_team(a, C, M, labels, ws, L, W, H, g, p);
         a.T = TW;
         a.NT = NT;
         a.nbands = (H + NT - 1) / NT;
@@ -429,7 +567,7 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
         // one column apart, so a short ring suffices and stays in L2; otherwise
         // the depth that lets the first resident band finish its row
         {
-            const int occ = edp_pass_line_occupancy(P->Q0, P->Q1, p->l1, split, 32 * TW * NT, P->smem);
+            const int occ = edp_pass_line_occupancy(P->Q0, P->Q1, p->l1, 32 * TW * NT, P->smem);
             const bool all_resident = a.nbands <= std::max(1, occ) * sms;
             a.ring = all_resident ? std::min(kLineRingResident, team_ring(2 * W, kResidentMin))
                                   : team_ring(2 * W, kResidentMin);
@@ -549,6 +687,7 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
 // Control words that must start from zero before the first pass: status,
 // consumed-column and band counters, and the used hand-off records.
 size_t control_bytes(const SolvePlan &P, int W, int Q) {
+    if (P.split) return P.L.ll;  // plain values, published by the flags
     return P.r1 ? P.L.ll + (size_t)P.nbands * 2 * W * Q * 8 : P.L.ll + (size_t)P.nbands * P.ta.ring * P.L.Qm * 8;
 }
 
@@ -607,7 +746,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     int rc = plan_solve(C, W, H, g, p, labels, ws, &P);
     if (rc) return rc;
     if (fi) {
-        if (!P.line || !P.split) return EDP_ERR_UNSUPPORTED;
+        if (!P.split) return EDP_ERR_UNSUPPORTED;
         P.ta.fI0 = fi->I0;
         P.ta.fI1 = fi->I1;
         P.ta.fpitch = fi->pitch;
@@ -618,7 +757,8 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
         P.ta.fcmax = fi->cmax;
         P.ta.fl2 = fi->l2;
     }
-    if (wh && !P.r1 && !P.line && !P.ta.lean) return EDP_ERR_UNSUPPORTED;  // not the lane-group form
+    // per-edge multipliers: not the spaces of the lane-group form
+    if (wh && !P.r1 && !(P.split ? lean_space(g) : P.line || P.ta.lean)) return EDP_ERR_UNSUPPORTED;
     P.o.wh = P.ta.wh = wh;
     P.o.wv = P.ta.wv = wv;
     if ((rc = cuda_status(cudaMemsetAsync(ws, 0, control_bytes(P, W, g.Q), st)))) return rc;
@@ -626,8 +766,13 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     bool resident;  // every row band has a block at once
-    if (P.line) {
-        const int occ = std::max(1, edp_pass_line_occupancy(P.Q0, P.Q1, P.ta.l1, P.split, P.threads, P.smem));
+    if (P.split) {
+        grid_t = std::max(1, edp_pass_line2_occupancy(P.build, P.threads, P.smem)) * sms;
+        // the items of both passes of a pair fill the blocks back to back, which
+        // saves one drain of the resident rows per pair
+        resident = P.nbands <= 4 * grid_t;
+    } else if (P.line) {
+        const int occ = std::max(1, edp_pass_line_occupancy(P.Q0, P.Q1, P.ta.l1, P.threads, P.smem));
         grid_t = std::min(P.nbands, occ * sms);
         if (grid_t < P.nbands && team_ring(2 * W, grid_t) > P.ta.ring) return EDP_ERR_UNSUPPORTED;
         resident = grid_t >= P.nbands;
@@ -658,7 +803,17 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
             const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
             if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)
                 return EDP_ERR_CUDA;
-            if (P.line) {
+            if (P.split) {
+                TeamArgs a = P.ta;
+                const int slot = it * 4 + set_launch(a, it, k, p->iters, pairs);
+                a.cons = reinterpret_cast<unsigned *>(ws + P.L.lcons) + (size_t)slot * H * kLineFlagStride;
+                a.rflag = reinterpret_cast<unsigned *>(ws + P.L.lflag) + (size_t)slot * H * kLineFlagStride;
+                a.hold_band = g_hold_band;
+                a.band_counter = reinterpret_cast<unsigned *>(ws + P.L.counters) + slot;
+                a.grid = std::min(grid_t, P.nbands * (pairs ? 2 : 1));
+                a.trace = trace;
+                if (launch_edp_pass_line2(a, P.build, P.threads, P.smem, st)) return EDP_ERR_CUDA;
+            } else if (P.line) {
                 TeamArgs a = P.ta;
                 const int slot = it * 4 + set_launch(a, it, k, p->iters, pairs);
                 a.cons = reinterpret_cast<unsigned *>(ws + P.L.lcons) + (size_t)slot * H * kLineFlagStride;
@@ -668,7 +823,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
                 a.band_counter = reinterpret_cast<unsigned *>(ws + P.L.counters) + slot;
                 a.grid = grid_t;
                 a.trace = trace;
-                if (launch_edp_pass_line(a, P.Q0, P.Q1, P.split, P.threads, P.smem, st)) return EDP_ERR_CUDA;
+                if (launch_edp_pass_line(a, P.Q0, P.Q1, P.threads, P.smem, st)) return EDP_ERR_CUDA;
             } else if (P.r1) {
                 PassR1Args a = P.o;
                 const int slot = it * 4 + set_launch(a, it, k, p->iters, pairs);  // counters of the first pass
@@ -1106,7 +1261,7 @@ int edp_solve_images(const uint8_t *I0, const uint8_t *I1, const uint8_t *I2, in
     bool fuse = false;
     if (g_fused_cost && params->cost_mode == 0 && space->R == 2) {
         SolvePlan P;
-        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.line && P.split;
+        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.split;
     }
     const FusedImages fi = fused_images(I0, I1, pitch, space, params);
     if (!fuse && (rc = run_cost(I0, I1, I2, W, H, pitch, space, params, g.Q, C, st))) return rc;
@@ -1422,6 +1577,51 @@ int edp_cost_window(const uint8_t *I0, const uint8_t *I1, const uint8_t *I2, int
     return launch_cost_window(a, centre, win, (cudaStream_t)stream) ? EDP_ERR_CUDA : EDP_OK;
 }
 
+namespace {
+// The passes of a windowed solve on the box kernel (edp_pass_win.cu); a holds
+// the problem.  EDP_ERR_UNSUPPORTED: no launch shape (nothing was launched).
+int run_windowed(TeamArgs a, const SolveLayout &L, unsigned char *w, int iters, int sms, cudaStream_t st) {
+    const int W = a.W, H = a.H;
+    a.nbuf = 4;
+    a.T = 1;
+    // rows per block (a compute and four copy warps each): enough blocks for the
+    // SMs first, then few hand-offs between blocks
+    int NT = g_tune_rb > 0 ? g_tune_rb : std::max(1, (H + sms - 1) / sms);
+    NT = std::max(1, std::min(std::min(NT, 5), H));
+    a.NT = NT;
+    const int threads = pass_line2_threads(NT, 1);
+    const size_t smem = pass_win_smem(NT, L.Qm, a.nbuf);
+    if (smem > (size_t)kMaxSmem) return EDP_ERR_UNSUPPORTED;
+    const int occ = edp_pass_win_occupancy(a.win, threads, smem);
+    a.nbands = (H + NT - 1) / NT;
+    a.ring = a.nbuf + (a.nbands <= occ * sms ? 8 : team_ring(W, std::max(1, occ * sms)));
+    if (occ < 1 || a.ring > 2 * team_ring(2 * W, kResidentMin)) return EDP_ERR_UNSUPPORTED;
+    int rc;
+    if ((rc = cuda_status(cudaMemsetAsync(w, 0, L.ll, st)))) return rc;
+    const bool pairs = pairs_for(a.nbands <= 4 * occ * sms);
+    const int per_it = pairs ? 2 : 4;
+    a.grid = std::min(a.nbands * (pairs ? 2 : 1), occ * sms);
+    g_last_launches = per_it * iters;
+    g_last_kernel = "edp_pass_line2_kernel";
+    for (int it = 0; it < iters; ++it)
+        for (int k = 0; k < per_it; ++k) {
+            const int launch = it * per_it + k;
+            TeamArgs b = a;
+            const int slot = it * 4 + set_launch(b, it, k, iters, pairs);
+            b.cons = reinterpret_cast<unsigned *>(w + L.lcons) + (size_t)slot * H * kLineFlagStride;
+            b.rflag = reinterpret_cast<unsigned *>(w + L.lflag) + (size_t)slot * H * kLineFlagStride;
+            b.band_counter = reinterpret_cast<unsigned *>(w + L.counters) + slot;
+            const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
+            if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)
+                return EDP_ERR_CUDA;
+            if (launch_edp_pass_win(b, threads, smem, st)) return EDP_ERR_CUDA;
+            if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch + 1], st) != cudaSuccess)
+                return EDP_ERR_CUDA;
+        }
+    return EDP_OK;
+}
+}  // namespace
+
 int edp_solve_windowed(const int32_t *Cw, const int32_t *centre, int win, int W, int H,
                        const edp_label_space *space, const edp_params *params, int32_t *labels, void *ws,
                        size_t ws_bytes, edp_stream_t stream) {
@@ -1437,8 +1637,7 @@ int edp_solve_windowed(const int32_t *Cw, const int32_t *centre, int win, int W,
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char *w = static_cast<unsigned char *>(ws);
     const int Qw = space->R == 2 ? win * win : win;
-    // the multi-axis pass kernel in its windowed form: one warp per row, the
-    // workspace laid out as edp_solve's with Q = Qw
+    // one warp per row, the workspace laid out as edp_solve's with Q = Qw
     const SolveLayout L = solve_layout(W, H, Qw, space->R, params->iters);
     TeamArgs a;
     memset(&a, 0, sizeof a);
@@ -1455,6 +1654,23 @@ int edp_solve_windowed(const int32_t *Cw, const int32_t *centre, int win, int W,
     a.lam = params->lambda;
     a.capv = (int)cap_value(params);
     a.mode = params->prior_mode;
+    a.win = win;
+    a.l1 = params->l1;
+    a.g = params->g;
+    a.centre = centre;
+    a.Q0w = space->Q[0];
+    a.Q1w = space->Q[1];
+    a.spin_limit = g_spin_limit;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    // two axes, linear prior: the box kernel in the split line kernel's frame
+    if (space->R == 2 && params->l1 == 1 && pass_win_built(win) && (reinterpret_cast<uintptr_t>(Cw) & 15) == 0) {
+        const int rc2 = run_windowed(a, L, w, params->iters, sms, st);
+        if (rc2 != EDP_ERR_UNSUPPORTED) return rc2;
+    }
+    // otherwise the multi-axis pass kernel in its windowed form
     a.T = 1;
     int NT = g_tune_rb > 0 ? g_tune_rb : 8;
     NT = std::max(1, std::min(NT, std::min(8, H)));  // the windowed builds take <= 256 threads
@@ -1466,19 +1682,9 @@ int edp_solve_windowed(const int32_t *Cw, const int32_t *centre, int win, int W,
     if (smem > (size_t)kMaxSmem) return EDP_ERR_UNSUPPORTED;
     a.NT = NT;
     a.ring = team_ring(2 * W, kResidentMin);
-    a.win = win;
-    a.l1 = params->l1;
-    a.g = params->g;
-    a.centre = centre;
-    a.Q0w = space->Q[0];
-    a.Q1w = space->Q[1];
     a.em = params->l1;  // the windowed build of this prior power
     a.nbands = (H + NT - 1) / NT;
-    a.spin_limit = g_spin_limit;
     const int laps = (W + a.ring - 1) / a.ring;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int occ = std::max(1, edp_pass_team_occupancy(a.em, 0, 1, 32 * NT, smem));
     a.grid = std::min(a.nbands, occ * sms);
     if (a.grid < a.nbands && team_ring(2 * W, a.grid) > a.ring) return EDP_ERR_UNSUPPORTED;

@@ -1,0 +1,9 @@
+// edp_pass_line2_e.cu -- builds of the split line kernel (see edp_pass_line2.cu).
+#include "line2_kernel.cuh"
+
+namespace edp {
+
+void *line2_k9(bool fused) { return line2_kernel<Build<Cut<8, 4>, Cut<4, 4>, Cut<0, 0>, false>, false>(fused); }
+void *line2_k10(bool fused) { return line2_kernel<Build<Cut<8, 4>, Cut<4, 8>, Cut<0, 0>, false>, false>(fused); }
+
+}  // namespace edp

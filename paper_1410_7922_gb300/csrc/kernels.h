@@ -39,6 +39,13 @@ struct TeamAxis {
     int kc;       // lanes of carry in the truncated sweeps
     int rounds;   // line groups per lane, ceil(nlines * G / (32 T))
 };
+// lines cut into segments held by several lanes (pass_line2.cuh)
+struct SegAxis {
+    int S;        // segments (lanes) per line
+    int lpw;      // lines per warp, 32 / S
+    int nf;       // segments that hold E labels (the others hold E - 1)
+    int kc;       // segments of carry in the truncated sweeps
+};
 struct TeamArgs {
     const int *C;           // [H][W][Q]
     int *M[4];              // [H][W][Qm] messages into each pixel from +x, -x, +y, -y
@@ -50,6 +57,7 @@ struct TeamArgs {
     int *status;
     int W, H, Q, Qm, R;     // Qm: message stride, Q rounded up to a multiple of 4
     TeamAxis ax[3];
+    SegAxis seg[3];         // split line kernel
     int lam, capv, mode;    // mode 0 joint, 1 per axis truncation
     const uint8_t *wh, *wv; // optional [H][W] prior multipliers of the edges (x,y)-(x+1,y), (x,y)-(x,y+1) (lean form)
     int l1, g;              // prior power (1: linear sweeps, 2: quadratic taps, lean / windowed forms) and truncation
@@ -80,16 +88,37 @@ size_t pass_team_smem(int NT, int Qm, int R, int nbuf, int kmb);
 
 // one EDP scan pass, two label axes, one label line per lane (edp_pass_line.cu);
 // uses TeamArgs with T = warps per row, NT = rows per block
-// split: the form with each label line shared by two lanes (pass_line2.cuh)
 bool pass_line_built(int Q0, int Q1, int l1);
-bool pass_line_split_built(int Q0, int Q1, int l1);
-int pass_line_split_max_lambda();
-int pass_line_warps(int Q0, int Q1, bool split);
-size_t pass_line_smem(int NT, int Q0, int Q1, bool split);
-int edp_pass_line_occupancy(int Q0, int Q1, int l1, bool split, int threads, size_t smem);
-int launch_edp_pass_line(const TeamArgs &a, int Q0, int Q1, bool split, int threads, size_t smem, cudaStream_t st);
+int pass_line_warps(int Q0, int Q1);
+size_t pass_line_smem(int NT, int Q0, int Q1);
+int edp_pass_line_occupancy(int Q0, int Q1, int l1, int threads, size_t smem);
+int launch_edp_pass_line(const TeamArgs &a, int Q0, int Q1, int threads, size_t smem, cudaStream_t st);
+// one EDP scan pass (or paired sweep), two or three label axes, each label
+// line split over lanes (edp_pass_line2.cu); T = compute warps per row,
+// NT = rows per block, nbuf stages
+int pass_line2_max_lambda();
+struct Line2Build {
+    int S[3], E[3];          // segments per line and labels per lane of each axis (S = 0: no such axis)
+    bool exact;              // lines of exactly E or E - 1 labels per segment, else any that fit
+    int threads;             // bound of a block
+    void *(*kernel)(bool fused);
+};
+int pass_line2_builds();
+const Line2Build &pass_line2_build(int b);
+int pass_line2_max_warps();
+int pass_line2_threads(int NT, int T);
+size_t pass_line2_smem(int NT, int Qm, int nst);
+int edp_pass_line2_occupancy(int build, int threads, size_t smem);
+int launch_edp_pass_line2(const TeamArgs &a, int build, int threads, size_t smem, cudaStream_t st);
+// the same on per-pixel label boxes of win x win labels (edp_pass_win.cu), one
+// compute warp per row
+bool pass_win_built(int n);
+size_t pass_win_smem(int NT, int Qm, int nst);
+int edp_pass_win_occupancy(int n, int threads, size_t smem);
+int launch_edp_pass_win(const TeamArgs &a, int threads, size_t smem, cudaStream_t st);
 // per-band stride of the line kernels' record flags and consumed counters
-// (one per warp of the producing / consuming team)
+// (one-lane form: one per warp of the producing / consuming team; split form:
+// flags of the even and odd columns, [2] the row's finished copy warps)
 constexpr int kLineFlagStride = 8;
 
 // one EDP scan pass, one label axis, one warp per row (edp_pass_r1.cu)

@@ -1,83 +1,151 @@
-// pass_line2.cuh -- EDP scan pass for two-axis label spaces whose lines hold
-// 33 to 65 labels, each label line shared by two lanes.
+// pass_line2.cuh -- EDP scan pass for label spaces of two or three axes, each
+// label line shared by several lanes of a warp.
 //
-// Same messages, flags, pass schedule and hand-off protocol as
-// pass_line.cuh; what differs is that a line of L labels is split into a
-// first half of 32 labels and a second half of L - 32, held by lanes l and
-// l + 16 of one warp (a warp serves 16 lines).  A lane loads, sums and
-// halves only its half of the line, so the per-lane state, the loads in
-// flight per lane and the dependent sweep chains are half as long.
+// Same messages, flags and pass schedule as pass_team.cuh (M[k] at pixel x
+// holds m_k(x) = M(floor(S_k(x_k) / 2)); a pass updates the sums a, b from
+// m_a, m_b of this pass and m_c, m_d of earlier ones).  A pass is a wavefront,
+// so what bounds it is the time of one column step of one row; this kernel
+// spreads a row over as many warps as its labels fill, keeps every memory
+// access of the step in shared memory, and moves all global data with bulk
+// asynchronous copies issued by warps that do nothing else.
 //
-// The LRMS sweeps of Sec. 3.2 over a split line.  The backward sweep
-// (Eq. L_dec5) is the minimum over j >= i of h[j] + lambda (j - i), so after
-// each half ran it on its own the first half only misses the sources of the
-// second half, which all reach label i through label 32:
-//     b[i] = min(b_1st[i], b[32] + lambda (32 - i))     (i < 32),
-// and b[32] is the second half's own first value.  Likewise the forward
-// sweep (Eq. L_dec3) over b, f[i] = min over j <= i of b[j] + lambda (i - j),
-// completes the second half with the first half's last value:
-//     f[i] = min(f_2nd[i], f[31] + lambda (i - 31))     (i >= 32).
-// Each completion is one shuffle and a set of independent add-mins.  The
-// products lambda k (k <= 33) stay below 2^30, which the planner checks
-// before it picks this kernel.
+// Roles.  A block holds NT teams (NT consecutive rows, one band).  A team has
+// T compute warps and four copy warps (one lane each):
+//   stage  copies C, m_c, m_d of the columns ahead into a ring of nst stages;
+//   above  (first row of a band) copies m_b of the columns the row above has
+//          published into the same stages;
+//   out 0, out 1  (even / odd columns) copy the finished m_a and m_b to the
+//          message arrays and, for the last row of a band, publish the column.
+// They meet in mbarriers: load[stage] completes when a column's copies (C, m_c,
+// m_d; m_b of `above`) have landed, ready[stage] when its output buffers have
+// been shipped and, below another team, that team's warps have written m_b;
+// empty[stage] when every compute warp has read the inputs; outf[p] when every
+// compute warp has written its outputs.
 //
-// Shared memory: the [LA][LB] transposition buffers (X_a and the two mailbox
-// slots of each team) are stored as four quadrants (i < 32 or not, k < 32 or
-// not) with a row pitch of 33 and bases placed so that, in both phases, the
-// 16 lanes of the first halves and the 16 of the second halves fall on
-// different banks.
+// A column step of the compute warps:
+//   phase 0   the halved sums of Eq. DP_2D_base on lines of axis 0, both
+//             vectors in the same lane (the five inputs are read once), the
+//             min search along axis 0, results to X_a (next buffer) and X_b;
+//   barrier;  phases 1 .. R-1: the same along axes 1, 2 in place, one vector
+//             per warp (a barrier between them); the last one leaves m_a in X_a
+//             and m_b in the stage of the row below (or in X_b, shipped by `out`);
+//   barrier.
+// The min search is separable, so the order of the axes changes no value.
 //
-// Between blocks the hand-off ships the mailbox slot as it is: a ring of
-// slot images in global memory (the quadrant layout, plain 32-bit values,
-// no {value, tag} words).  Each thread of the last row of a block copies its
-// 16-byte chunks of the outgoing slot there, then one lane per warp
-// publishes them with a release store of the warp's flag at GPU scope; the
-// same thread of the first row of the block below acquires that flag and
-// copies the same chunks into its own, otherwise unused, mailbox slot with
-// asynchronous copies (no registers in flight), and after a team barrier
-// the row runs as every other row.
+// A line of L labels is cut into S segments (S a power of two) of e = ceil(L / S)
+// or e - 1 labels; lane k * lpw + l of a warp holds segment k of the warp's line
+// l (lpw = 32 / S lines per warp), so neighbouring lanes read neighbouring
+// lines (odd strides: distinct banks).  Per segment the forward and the
+// backward sweep (Eq. L_dec3, Eq. L_dec5) run on the lane's own labels; the
+// values at the segment's ends travel by one shuffle per direction, kc
+// segments far, and complete the labels they can still improve: a source
+// g or more labels away costs at least the clip value applied afterwards
+// (Sec. 3.1), so nothing beyond is needed.
+//
+// A column step is a few hundred instructions in a row, run by a few warps per
+// scheduler, so what costs is not the arithmetic but every taken branch and
+// every load from the parameter block (tens of cycles each).  Hence one build
+// per cut of the axes (labels per lane as constants, EXACT where the cut
+// matches e), the truncation mode and the last pass as separate copies of the
+// column loop, and predicated single instructions instead of short branches.
+// (A build that picked the cut at run time took 2.2 us a column at 33 x 33
+// labels.)
+//
+// Between bands.  The messages m_b are in global memory either way: in the
+// passes that keep them, in the message array M[b] itself; in the others in a
+// ring of `ring` columns per band that stays in L2.  The producing `out` warp
+// publishes a column when its copies have completed (release at GPU scope);
+// the `above` warp of the next band acquires it and copies it in.  A ring slot
+// is written again once the consumer has counted its column (cons).
+//
+// Work items.  A launch holds one pass, or two that share the vertical
+// direction (A.pair: P1 then P2, or P3 then P4) as items (half, band) claimed
+// in order.  Row y of the second half needs row y of the first half complete
+// (its m_a are this half's m_c) and its own half's row above, both claimed
+// earlier, so a block never waits for an item that nobody runs; the second
+// half starts without draining the first.
 #pragma once
-#include "pass_line.cuh"
+#include <type_traits>
+
+#include "common.cuh"
+#include "kernels.h"
 
 namespace edp {
 namespace line2 {
 
-constexpr int kPQ = 33;        // row pitch of a quadrant (odd)
-constexpr int kMaxWarps = 8;   // warps per team (16 lines each)
-constexpr int kMaxThreads = 640;
-// control ints of one team: [0, 8) produced columns per warp, [8, 16)
-// consumed columns per warp, [16, 24) / [24, 32) warp minima of the halved
-// S_a / S_b sums, [32, 48) warp argmin keys (eight 64-bit); 64 in all, so
-// that the buffers after it start on bank 0
-constexpr int kCtl = 64;
-
-// smallest y >= x with y = r (mod 32)
-__host__ __device__ constexpr int up32(int x, int r) { return x + ((r - x) % 32 + 32) % 32; }
-// base of quadrant (hi, hk) of an [LA][LB] buffer (rows i in [32 hi, ...),
-// columns k in [32 hk, ...)); bases 0, 16, 16, 0 (mod 32)
-__host__ __device__ constexpr int qbase(int LA, int hi, int hk) {
-    return hi == 0 ? (hk == 0 ? 0 : up32(32 * kPQ, 16))
-                   : (hk == 0 ? up32(up32(32 * kPQ, 16) + 32 * kPQ, 16)
-                              : up32(up32(up32(32 * kPQ, 16) + 32 * kPQ, 16) + (LA - 32) * kPQ, 0));
-}
-__host__ __device__ constexpr int buf_ints(int LA) { return up32(qbase(LA, 1, 1) + (LA - 32) * kPQ, 0); }
-// ints of shared memory of one team: control, X_a, two mailbox slots
-__host__ __device__ constexpr size_t team_ints(int LA) { return kCtl + 3 * (size_t)buf_ints(LA); }
-// the planner's bound on the prior weight (the completions add lambda * 33)
+constexpr unsigned kFull = 0xffffffffu;
+constexpr int kCopyWarps = 4;     // stage, above, out 0, out 1
+constexpr int kMaxT = 24;         // compute warps of a team
+constexpr int kMaxThreads = 896;  // of a block: 72 registers a thread
+constexpr int kMaxStages = 4;
+// control ints of one team: mbarriers [0, 28), columns issued by `stage` and
+// `above` (an aborted item's, [28, 30)), abort flag [30], warp minima [32, 80), warp argmin
+// values and labels [80, 128)
+constexpr int kCtlInts = 128;
+// the planner's bound on the prior weight (sweeps add up to 33 lambda to kBig)
 constexpr int kMaxLambda = (1 << 30) / 34;
 
-// Global loads as volatile asm: issued in program order, so that a batch is
-// in flight as a whole (the compiler does not sink them to their uses)
-__device__ __forceinline__ int ld_cs(const int *p) {
+// a stage: C (and 4 ints of slack for its 16-byte alignment), m_c, m_d, m_b
+__host__ __device__ inline size_t stage_ints(int Qm) { return 4 * (size_t)Qm + 4; }
+// ints of one team: stages, X_a and X_b (two each), `extra` further vectors,
+// control
+__host__ __device__ inline size_t team_ints(int Qm, int nst, int extra) {
+    return nst * stage_ints(Qm) + (4 + extra) * (size_t)Qm + kCtlInts;
+}
+
+__device__ __forceinline__ unsigned saddr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ int lds(unsigned a) {
     int v;
-    asm volatile("ld.global.cs.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
     return v;
 }
-__device__ __forceinline__ int ld_cg(const int *p) {
-    int v;
-    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p));
-    return v;
+__device__ __forceinline__ void sts(unsigned a, int v) { asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+
+__device__ __forceinline__ void mbar_init(unsigned b, unsigned count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(unsigned b) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(b) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(unsigned b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_tx(unsigned b, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned b, unsigned parity) {
+    unsigned r;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"(b), "r"(parity)
+        : "memory");
+    return r != 0;
+}
+// bounded wait for the completion of a phase; false when it ran out or the
+// block is aborting
+__device__ __forceinline__ bool mbar_wait(unsigned b, unsigned parity, long long limit, volatile int *s_abort) {
+    if (mbar_try(b, parity)) return true;
+    for (long long n = 0; n < limit; ++n) {
+        if (mbar_try(b, parity)) return true;
+        if (*s_abort) return false;
+    }
+    return false;
+}
+// bulk copies (16-byte aligned addresses and sizes)
+__device__ __forceinline__ void bulk_load(unsigned dst, const int *src, unsigned bytes, unsigned mbar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(mbar)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_store(int *dst, unsigned src, unsigned bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ unsigned ld_acq_gpu(const unsigned *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -86,441 +154,690 @@ __device__ __forceinline__ unsigned ld_acq_gpu(const unsigned *p) {
 __device__ __forceinline__ void st_rel_gpu(unsigned *p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-
-// LRMS sweeps of one split line, in place: the lane holds labels [32 hf,
-// 32 hf + n) of the line in h[0, n), kBig above; its partner lane (lane ^ 16)
-// the other half.  Then the clip.  mask: the lanes of the warp that call it
-// (partners together).
-template <int N>
-__device__ __forceinline__ void split_sweeps(int (&h)[N], const bool lo, const int lam, const int clip,
-                                             const unsigned mask) {
-#pragma unroll
-    for (int i = N - 2; i >= 0; --i) h[i] = __viaddmin_s32(h[i + 1], lam, h[i]);
-    const int cb = __shfl_xor_sync(mask, h[0], 16);  // b[32], from the second half
-    if (lo) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) h[i] = __viaddmin_s32(cb, lam * (32 - i), h[i]);
+__device__ __forceinline__ void add_rel_gpu(unsigned *p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint2 ld_acq_gpu2(const unsigned *p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return make_uint2((unsigned)v, (unsigned)(v >> 32));
+}
+__device__ __forceinline__ void st_relaxed_gpu(unsigned *p, unsigned v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// bounded poll of a counter of another block
+__device__ __forceinline__ bool wait_count(const unsigned *p, int need, long long limit, volatile int *s_abort,
+                                           const int *status) {
+    for (long long n = 0; n <= limit; ++n) {
+        if ((int)ld_acq_gpu(p) >= need) return true;
+        if (*s_abort || ((n & 63) == 63 && *(volatile const int *)status != 0)) return false;
+        __nanosleep(20);
     }
-#pragma unroll
-    for (int i = 1; i < N; ++i) h[i] = __viaddmin_s32(h[i - 1], lam, h[i]);
-    const int cf = __shfl_xor_sync(mask, h[31], 16);  // f[31], from the first half
-    if (!lo) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) h[i] = __viaddmin_s32(cf, lam * (i + 1), h[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < N; ++i) h[i] = min(h[i], clip);
+    return false;
+}
+// barriers of the T compute warps of a team; the second also returns the OR
+// of pred over them
+__device__ __forceinline__ void team_sync(int tm, int T) {
+    asm volatile("barrier.sync %0, %1;" ::"r"(tm + 1), "r"(32 * T) : "memory");
+}
+__device__ __forceinline__ bool team_sync_or(int tm, int T, bool pred) {
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.s32 p, %1, 0;\n\t"
+        "barrier.red.or.pred q, %2, %3, p;\n\t"
+        "selp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((int)pred), "r"(tm + 1), "r"(32 * T)
+        : "memory");
+    return r != 0;
 }
 
-// Phase A loads of one half label column of one pixel: C straight into hv
-// (all of it in flight at once, in the registers the line needs anyway),
-// the old messages m_c and m_d (global, coalesced across the 16 lanes of
-// each half) in batches of CH labels one batch ahead of the arithmetic, m_a
-// from xa and m_b from xb (shared memory, stride kPQ); the messages this
-// pixel received written to the message arrays, and the two halved sums of
-// Eq. DP_2D_base: S_a into hv (kBig above the lane's n labels), S_b over m_b
-// in xb.  Two batches are in flight ahead of the arithmetic.
-template <int N, int LB, int CH>
-__device__ __forceinline__ void issue_batch(const int *__restrict__ Mcp, const int *__restrict__ Mdp,
-                                            const bool c_ok, const bool d_ok, const int n, const int b,
-                                            int (&mcv)[CH], int (&mdv)[CH]) {
-#pragma unroll
-    for (int jj = 0; jj < CH; ++jj) {
-        const int i = b * CH + jj;
-        if (i < N && i < n) {
-            const int o = i * LB;
-            mcv[jj] = c_ok ? ld_cs(Mcp + o) : 0;
-            mdv[jj] = d_ok ? ld_cs(Mdp + o) : 0;
-        }
-    }
-}
-// The pair cost of Eq. Cost_value for the lane's half column, computed from
-// the images: label i of the half has I1 row ys0 + t1 i at column col (the
-// lane's axis-0 offset); C = cmax outside the image, else
-// min(|I1 - I0(x)|^l2, cmax) -- the same values the cost kernels store.
-struct FusedCost {
-    const uint8_t *col;  // I1 + the lane's column (read only when col_ok)
-    bool col_ok;
-    int ys0, t1, H, pitch, i0, cmax, l2;
-};
-template <int N, int LB, int CH, bool FUSED>
-__device__ __forceinline__ void front_load(const int *__restrict__ Cp, const FusedCost &fc,
-                                           const int *__restrict__ Mcp, const int *__restrict__ Mdp,
-                                           const bool c_ok, const bool d_ok, const int n, int (&hv)[N],
-                                           int (&mcv)[2][CH], int (&mdv)[2][CH]) {
-    constexpr int NB = (N + CH - 1) / CH;
-    if constexpr (FUSED) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            if (i < n) {
-                const int ys = fc.ys0 + fc.t1 * i;
-                int c = fc.cmax;
-                if (fc.col_ok && (unsigned)ys < (unsigned)fc.H) {
-                    const int d = abs((int)fc.col[(size_t)ys * fc.pitch] - fc.i0);
-                    c = min(fc.l2 == 1 ? d : d * d, fc.cmax);
-                }
-                hv[i] = c;
-            } else {
-                hv[i] = kBig;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; ++i) hv[i] = i < n ? ld_cs(Cp + i * LB) : kBig;
-    }
-    issue_batch<N, LB, CH>(Mcp, Mdp, c_ok, d_ok, n, 0, mcv[0], mdv[0]);
-    if (NB > 1) issue_batch<N, LB, CH>(Mcp, Mdp, c_ok, d_ok, n, 1, mcv[1], mdv[1]);
-}
-template <int N, int LB, int CH, bool FUSED>
-__device__ __forceinline__ void half_load(const int *__restrict__ Cp, const FusedCost &fc, const int *__restrict__ Mcp,
-                                          const int *__restrict__ Mdp, int *__restrict__ Map,
-                                          int *__restrict__ Mbp, const int *__restrict__ xa, int *__restrict__ xb,
-                                          const bool c_ok, const bool d_ok, const bool has_ma, const bool mbox,
-                                          const bool st_a, const bool st_b, const bool fin, const int n,
-                                          const int q0, int (&hv)[N], int &lmin_a, int &lmin_b,
-                                          unsigned long long &key) {
-    constexpr int NB = (N + CH - 1) / CH;
-    int mcv[2][CH], mdv[2][CH];
-    front_load<N, LB, CH, FUSED>(Cp, fc, Mcp, Mdp, c_ok, d_ok, n, hv, mcv, mdv);
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-        const int k = b & 1;
-#pragma unroll
-        for (int jj = 0; jj < CH; ++jj) {
-            const int i = b * CH + jj;
-            if (i < N && i < n) {
-                const int o = i * LB;
-                const int mc = mcv[k][jj], md = mdv[k][jj];
-                const int ma = has_ma ? xa[i * kPQ] : 0;
-                const int mb = mbox ? xb[i * kPQ] : 0;
-                if (st_a) __stcs(Map + o, ma);
-                if (st_b) __stcs(Mbp + o, mb);
-                const int t = hv[i] + ma + mb, e = md - mc;
-                const int ha = floor_half(t + e), hb = floor_half(t - e);
-                if (fin) key = min(key, line::argmin_key(t + mc + md, q0 + o));
-                hv[i] = ha;
-                xb[i * kPQ] = hb;
-                lmin_a = min(lmin_a, ha);
-                lmin_b = min(lmin_b, hb);
-            }
-        }
-        // the batch after next, into the registers just consumed
-        if (b + 2 < NB) issue_batch<N, LB, CH>(Mcp, Mdp, c_ok, d_ok, n, b + 2, mcv[k], mdv[k]);
-    }
-}
-
-// 16-byte asynchronous copy global -> shared (L2 only), and the wait for
-// this thread's copies
-__device__ __forceinline__ void cp_async16(int *sdst, const int *gsrc) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(sdst)),
-                 "l"(gsrc)
+// predicated single instructions
+__device__ __forceinline__ void sts_if(bool p, unsigned a, int v) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.s32 [%0], %1;\n\t}" ::"r"(a), "r"(v),
+                 "r"((int)p)
                  : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+__device__ __forceinline__ void mbar_arrive_if(bool p, unsigned b) {
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(b),
+                 "r"((int)p)
+                 : "memory");
+}
+
+// The cut of one axis: S segments per line, at most E labels each.
+template <int S_, int E_>
+struct Cut {
+    static constexpr int S = S_, E = E_, lpw = 32 / S_;
+};
+
+// A lane's place on one axis.
+struct Seg {
+    int k;             // segment
+    int off;           // linear index of the segment's first label
+    int n;             // its labels
+    int gl, gr;        // labels between the segment's position 0 and the (virtual) last one of the segment before,
+                       // and between its (virtual) last one and position 0 of the segment after
+    bool on;           // the lane serves a line
+};
+// first position of segment k (the first nf segments hold e labels, the rest e - 1)
+__device__ __forceinline__ int seg_pos(int k, int e, int nf) { return k * (e - 1) + min(k, nf); }
+// the lane's place when the warp serves the lines from li0
+template <class C>
+__device__ __forceinline__ Seg seg_of(const SegAxis &G, const TeamAxis &X, int li0, int lane) {
+    Seg s;
+    s.k = lane / C::lpw;
+    const int li = li0 + lane - s.k * C::lpw;
+    s.on = li < X.nlines;
+    const int p = seg_pos(s.k, X.E, G.nf);
+    s.n = seg_pos(s.k + 1, X.E, G.nf) - p;
+    s.gl = p - seg_pos(s.k - 1, X.E, G.nf) - C::E + 1;
+    s.gr = s.n - C::E + 1;
+    s.off = 0;
+    if (s.on) {
+        // first label of line li
+        int f = li;
+        if (X.stride == 1)
+            f = li * X.L;
+        else if (li >= X.stride)
+            f = (li % X.stride) + (li / X.stride) * X.stride * X.L;
+        s.off = f + p * X.stride;
+    }
+    return s;
+}
+
+// The min search's constants of a pass: carries from kc segments; near: one
+// segment, and only the labels next to a boundary can improve (g <= 4).
+struct Dt {
+    int kc, e, nf;
+    bool near;
+};
+
+// Truncated L1 distance transform and clip of one vector's segment, in place
+// (positions n .. E - 1 hold kBig); cl is the clip value.  f, b: the lane's
+// own sweeps.
+template <class C, bool EXACT>
+__device__ __forceinline__ void seg_dt(int (&h)[C::E], const Seg &s, const Dt &D, const int lam, const int cl) {
+    constexpr int E = C::E;
+    int f[E], b[E];
+    f[0] = h[0];
+    b[E - 1] = h[E - 1];
+#pragma unroll
+    for (int i = 1; i < E; ++i) {
+        f[i] = __viaddmin_s32(f[i - 1], lam, h[i]);
+        b[E - 1 - i] = __viaddmin_s32(b[E - i], lam, h[E - 1 - i]);
+    }
+    if constexpr (C::S > 1) {
+        // carries: cf at position 0 of the segment, cb at position E - 1
+        const int F = f[E - 1], B = b[0];
+        int cf = __shfl_up_sync(kFull, F, C::lpw) + lam * s.gl, cb = __shfl_down_sync(kFull, B, C::lpw) + lam * s.gr;
+        cf = s.k > 0 ? cf : kBig;
+        cb = s.k + 1 < C::S ? cb : kBig;
+        // labels within 3 of the segment's ends, or all of them
+        constexpr int NF = EXACT && E > 3 ? 3 : E, NB = EXACT && E > 4 ? 4 : E;
+        if (__builtin_expect(!D.near, 0)) {
+#pragma unroll 1
+            for (int d = 2; d <= D.kc; ++d) {
+                const int uf = __shfl_up_sync(kFull, F, d * C::lpw), ub = __shfl_down_sync(kFull, B, d * C::lpw);
+                const int p = seg_pos(s.k, D.e, D.nf);
+                if (s.k >= d) cf = min(cf, uf + lam * (p - seg_pos(s.k - d, D.e, D.nf) - E + 1));
+                if (s.k + d < C::S) cb = min(cb, ub + lam * (seg_pos(s.k + d, D.e, D.nf) - p - E + 1));
+            }
+#pragma unroll
+            for (int i = NF; i < E; ++i) f[i] = __viaddmin_s32(cf, lam * i, f[i]);
+#pragma unroll
+            for (int i = 0; i < E - NB; ++i) b[i] = __viaddmin_s32(cb, lam * (E - 1 - i), b[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NF; ++i) f[i] = __viaddmin_s32(cf, lam * i, f[i]);
+#pragma unroll
+        for (int i = E - NB; i < E; ++i) b[i] = __viaddmin_s32(cb, lam * (E - 1 - i), b[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < E; ++i) h[i] = __vimin3_s32(f[i], b[i], cl);
+}
+
+// minimum over the line (every lane of the line gets it)
+template <class C>
+__device__ __forceinline__ int line_min(int m) {
+#pragma unroll
+    for (int d = C::lpw; d < 32; d <<= 1) m = min(m, __shfl_xor_sync(kFull, m, d));
+    return m;
+}
+
+// The pair cost of Eq. Cost_value of one label (two-axis spaces) from the
+// images, as the cost kernels store it.
+struct FusedPix {
+    int x, y, i0;  // pixel, I0(pixel)
+};
+__device__ __forceinline__ int fused_cost(const TeamArgs &A, const FusedPix &p, int q0, int q1) {
+    const int xs = p.x + A.fv0 + A.ft0 * q0, ys = p.y + A.fv1 + A.ft1 * q1;
+    if ((unsigned)xs >= (unsigned)A.W || (unsigned)ys >= (unsigned)A.H) return A.fcmax;
+    const int d = abs((int)A.fI1[(size_t)ys * A.fpitch + xs] - p.i0);
+    return min(A.fl2 == 1 ? d : d * d, A.fcmax);
+}
+
+// Phase 0: sums, halving, min search along axis 0 for both vectors.  C .. mb:
+// shared addresses of the inputs' label 0, xa / xb of the outputs'.  ja, jb:
+// minima of the halved sums (joint truncation); sv, sq: the marginal's lowest
+// value and label (FIN).
+struct In0 {
+    unsigned C, mc, md, ma, mb, xa, xb;
+    int lam_a, lam_b, cap_a, cap_b;
+    FusedPix fp;
+};
+template <class C, bool EXACT, bool FIN, bool PA, bool FUSED>
+__device__ __forceinline__ void phase0(const TeamArgs &A, const In0 &c, const Seg &s, const Dt &D, const int fq0,
+                                       const int fq1, int &ja, int &jb, int &sv, int &sq) {
+    constexpr int E = C::E;
+    const unsigned o = 4u * (unsigned)s.off;
+    int ha[E], hb[E];
+    int ma = kBig, mb = kBig;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const unsigned oi = o + 4 * i;
+        int cv;
+        if constexpr (FUSED)
+            cv = fused_cost(A, c.fp, fq0 + i, fq1);
+        else
+            cv = lds(c.C + oi);
+        const int mc = lds(c.mc + oi), md = lds(c.md + oi);
+        const int t = cv + lds(c.ma + oi) + lds(c.mb + oi);
+        ha[i] = floor_half(t + md - mc);
+        hb[i] = floor_half(t + mc - md);
+        if (FIN) {
+            const int so = t + mc + md;
+            if (s.on && i < s.n && so < sv) {
+                sv = so;
+                sq = s.off + i;
+            }
+        }
+        if ((!EXACT || i == E - 1) && i >= s.n) ha[i] = hb[i] = kBig;
+        ma = min(ma, ha[i]);
+        mb = min(mb, hb[i]);
+    }
+    int ca = kBig, cb = kBig;
+    if (PA) {
+        ca = line_min<C>(ma) + c.cap_a;
+        cb = line_min<C>(mb) + c.cap_b;
+    } else {
+        ja = min(ja, s.on ? ma : kBig);
+        jb = min(jb, s.on ? mb : kBig);
+    }
+    seg_dt<C, EXACT>(ha, s, D, c.lam_a, ca);
+    seg_dt<C, EXACT>(hb, s, D, c.lam_b, cb);
+    const int n = s.on ? s.n : 0;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const bool st = EXACT && i < E - 1 ? s.on : i < n;
+        sts_if(st, c.xa + o + 4 * i, ha[i]);
+        sts_if(st, c.xb + o + 4 * i, hb[i]);
+    }
+}
+
+// One line segment of a later phase: min search along the axis (neighbour
+// stride st4 bytes) of the values at src (label 0), results to dst; cl: the
+// clip value, or with PA what is added to the line's minimum.
+template <class C, bool EXACT, bool PA>
+__device__ __forceinline__ void phase_r(const Seg &s, const Dt &D, const unsigned src, const unsigned dst,
+                                        const unsigned st4, const int lam, const int cl) {
+    constexpr int E = C::E;
+    int h[E];
+    int m = kBig;
+    unsigned a = src + 4u * (unsigned)s.off;
+    const int last = s.n - 1;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        h[i] = lds(a);
+        if ((!EXACT || i == E - 1) && i > last) h[i] = kBig;
+        m = min(m, h[i]);
+        // past its last label a lane rereads it
+        if (EXACT ? i < E - 2 : i < last) a += st4;
+        if (EXACT && i == E - 2 && last == E - 1) a += st4;
+    }
+    seg_dt<C, EXACT>(h, s, D, lam, PA ? line_min<C>(m) + cl : cl);
+    a = dst + 4u * (unsigned)s.off;
+    const int n = s.on ? s.n : 0;
+#pragma unroll
+    for (int i = 0; i < E; ++i, a += st4) sts_if(EXACT && i < E - 1 ? s.on : i < n, a, h[i]);
+}
+
+static __device__ __noinline__ void timed_out(int *status, volatile int *s_abort) {
+    atomicCAS(status, 0, EDP_ERR_TIMEOUT_CODE);
+    *s_abort = 1;
+}
+
+// byte offsets of a team's mbarriers
+constexpr unsigned kLoadB = 0, kReadyB = 8 * kMaxStages, kEmptyB = 16 * kMaxStages, kOutB = 24 * kMaxStages;
+constexpr int kBars = (kOutB + 16) / 8;
+static_assert(kBars * 8 <= 112, "mbarriers of a team");
+
+struct Row {
+    int r, y, tm, wt, lane;
+    bool incx, incy, has_next, to_mbox, read_c, d_ok;
+};
+
+// arguments of a row's column loop: shared addresses of the zero vector, the
+// stages, X_a, X_b, the barriers, and of the team below the m_b of its first
+// stage and its ready barriers; the joint minima and argmin slots; the team's
+// abort flag
+#define EDP_ROW_ARGS                                                                                                   \
+    const TeamArgs &A, const Row &w, const unsigned zs, const unsigned st0, const unsigned xa0, const unsigned xb0,    \
+        const unsigned bars, const unsigned nx, const unsigned nx_ready, int *wmin, int *wkey, int *bad,               \
+        volatile int *s_abort
+template <class B, bool FIN, bool PA, bool FUSED>
+__device__ __forceinline__ void line2_row(EDP_ROW_ARGS);
+
+// A build: the cuts of the axes (C2::S = 0: two axes), exact or not.
+template <class C0_, class C1_, class C2_, bool EXACT_, int THREADS = kMaxThreads>
+struct Build {
+    using C0 = C0_;
+    using C1 = C1_;
+    using C2 = C2_;
+    static constexpr bool exact = EXACT_;
+    static constexpr int R = C2_::S > 0 ? 3 : 2;
+    static constexpr int threads = THREADS;  // bound of a block (registers)
+    template <bool FIN, bool PA, bool FUSED>
+    static __device__ __forceinline__ void row(EDP_ROW_ARGS) {
+        line2_row<Build, FIN, PA, FUSED>(A, w, zs, st0, xa0, xb0, bars, nx, nx_ready, wmin, wkey, bad, s_abort);
+    }
+    static constexpr int extra = 0;          // working vectors of a team beside X_a, X_b
+};
+template <>
+struct Cut<0, 0> {
+    static constexpr int S = 0, E = 1, lpw = 32;
+};
+
+// The column loop of one compute warp.
+template <class B, bool FIN, bool PA, bool FUSED>
+__device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
+    using C0 = typename B::C0;
+    using C1 = typename B::C1;
+    using C2 = typename B::C2;
+    constexpr bool X = B::exact;
+    constexpr int R = B::R;
+    const int W = A.W, Q = A.Q, T = A.T, tm = w.tm, wt = w.wt, lane = w.lane, y = w.y;
+    const unsigned vbytes = 4u * (unsigned)A.Qm, stb = 4u * (unsigned)stage_ints(A.Qm);
+    const unsigned omc = vbytes + 16, omd = 2 * vbytes + 16, omb = 3 * vbytes + 16;
+    const int n0 = (A.ax[0].nlines + C0::lpw - 1) / C0::lpw;  // warp rounds of the phases, per vector
+    const int n1 = (A.ax[1].nlines + C1::lpw - 1) / C1::lpw, n2 = (A.ax[2].nlines + C2::lpw - 1) / C2::lpw;
+    const Seg s0 = seg_of<C0>(A.seg[0], A.ax[0], wt * C0::lpw, lane);
+    const Seg s1 = seg_of<C1>(A.seg[1], A.ax[1], (wt >= n1 ? wt - n1 : wt) * C1::lpw, lane);
+    Seg s2 = s1;
+    if (R == 3) s2 = seg_of<C2>(A.seg[2], A.ax[2], (wt >= n2 ? wt - n2 : wt) * C2::lpw, lane);
+    const bool near = A.g <= 4;
+    const Dt d0{A.seg[0].kc, A.ax[0].E, A.seg[0].nf, near && A.seg[0].kc <= 1};
+    const Dt d1{A.seg[1].kc, A.ax[1].E, A.seg[1].nf, near && A.seg[1].kc <= 1};
+    const Dt d2{A.seg[2].kc, A.ax[2].E, A.seg[2].nf, near && A.seg[2].kc <= 1};
+    const unsigned st1 = 4u * (unsigned)A.ax[1].stride, st2 = 4u * (unsigned)A.ax[2].stride;
+    const unsigned send = 8u * (unsigned)A.nbuf;
+    const unsigned xa_sum = 2 * xa0 + vbytes, xb_sum = 2 * xb0 + vbytes;  // of the two buffers
+    unsigned sta = st0, sto = 0, stn = nx;  // stage of the column, its barriers, m_b in the stage of the row below
+    unsigned sph = 0, par = 0;
+    // the pixel's labels start this many ints into the 16-byte chunks copied
+    unsigned csh = FUSED ? 0u : (unsigned)((((size_t)y * W + (w.incx ? 0 : W - 1)) * Q) & 3);
+    const unsigned dcs = FUSED ? 0u : (unsigned)((w.incx ? Q : -Q) & 3);
+    In0 c;
+    c.lam_a = c.lam_b = A.lam;
+    c.cap_a = c.cap_b = A.capv;
+    c.ma = zs;
+    c.xa = xa0 + vbytes;
+    c.xb = xb0;
+#pragma unroll 1
+    for (int xs = 0; xs < W; ++xs) {
+        if (__builtin_expect(A.wh != nullptr, 0)) {  // per-edge multipliers of the two outgoing edges
+            const int x = w.incx ? xs : W - 1 - xs;
+            const int wa = xs + 1 < W ? __ldg(A.wh + (size_t)y * W + (w.incx ? x : x - 1)) : 1;
+            const int wb = w.has_next ? __ldg(A.wv + (size_t)(w.incy ? y : y - 1) * W + x) : 1;
+            c.lam_a = A.lam * wa;
+            c.cap_a = A.capv * wa;
+            c.lam_b = A.lam * wb;
+            c.cap_b = A.capv * wb;
+        }
+        c.C = sta + 4 * csh;
+        c.mc = w.read_c && xs + 1 < W ? sta + omc : zs;
+        c.md = w.d_ok ? sta + omd : zs;
+        c.mb = w.r > 0 ? sta + omb : zs;
+        if (FUSED) {
+            c.fp.x = w.incx ? xs : W - 1 - xs;
+            c.fp.y = y;
+            c.fp.i0 = A.fI0[(size_t)y * A.fpitch + c.fp.x];
+        }
+        bool ok = mbar_try(bars + kLoadB + sto, sph);
+        ok = mbar_try(bars + kReadyB + sto, sph) && ok;
+        if (__builtin_expect(!__all_sync(kFull, ok), 0)) {
+            ok = mbar_wait(bars + kLoadB + sto, sph, A.spin_limit, s_abort) &&
+                 mbar_wait(bars + kReadyB + sto, sph, A.spin_limit, s_abort);
+            if (!__all_sync(kFull, ok) && lane == 0) {
+                *bad = 1;
+                timed_out(A.status, s_abort);
+            }
+            __syncwarp();
+        }
+        int ja = kBig, jb = kBig, sv = 0x7fffffff, sq = 0x7fffffff;
+        if (wt < n0) {
+            phase0<C0, X, FIN, PA, FUSED>(A, c, s0, d0, seg_pos(s0.k, d0.e, d0.nf), wt * C0::lpw + (lane & (C0::lpw - 1)), ja,
+                                          jb, sv, sq);
+#pragma unroll 1
+            for (int t = wt + T; __builtin_expect(t < n0, 0); t += T) {
+                const Seg s = seg_of<C0>(A.seg[0], A.ax[0], t * C0::lpw, lane);
+                phase0<C0, X, FIN, PA, FUSED>(A, c, s, d0, seg_pos(s.k, d0.e, d0.nf),
+                                              t * C0::lpw + (lane & (C0::lpw - 1)), ja, jb, sv, sq);
+            }
+        }
+        if (FIN) {
+            const int v = __reduce_min_sync(kFull, sv);
+            const int q = __reduce_min_sync(kFull, sv == v ? sq : 0x7fffffff);
+            if (lane == 0) {
+                wkey[wt] = v;
+                wkey[kMaxT + wt] = q;
+            }
+        }
+        if (!PA) {
+            ja = __reduce_min_sync(kFull, ja);
+            jb = __reduce_min_sync(kFull, jb);
+            if (lane == 0) {
+                wmin[wt] = ja;
+                wmin[kMaxT + wt] = jb;
+            }
+        }
+        __syncwarp();
+        mbar_arrive_if(lane == 0, bars + kEmptyB + sto);  // this warp has read the column's inputs
+        team_sync(tm, T);
+        const int stop = lds(saddr(bad));  // written before this barrier only
+        if (FIN && wt == T - 1) {
+            const int v = lane < T ? wkey[lane] : 0x7fffffff, q = lane < T ? wkey[kMaxT + lane] : 0x7fffffff;
+            const int vm = __reduce_min_sync(kFull, v);
+            const int qm = __reduce_min_sync(kFull, v == vm ? q : 0x7fffffff);
+            if (lane == 0) A.labels[(size_t)y * W + (w.incx ? xs : W - 1 - xs)] = qm;
+        }
+        int ca = PA ? c.cap_a : kBig, cb = PA ? c.cap_b : kBig;
+        if (R == 3) {
+            auto mid = [&](const Seg &s, const bool vb) {
+                phase_r<C1, X, PA>(s, d1, vb ? c.xb : c.xa, vb ? c.xb : c.xa, st1, vb ? c.lam_b : c.lam_a, vb ? cb : ca);
+            };
+            if (wt < 2 * n1) {
+                mid(s1, wt >= n1);
+#pragma unroll 1
+                for (int t = wt + T; __builtin_expect(t < 2 * n1, 0); t += T)
+                    mid(seg_of<C1>(A.seg[1], A.ax[1], (t >= n1 ? t - n1 : t) * C1::lpw, lane), t >= n1);
+            }
+            team_sync(tm, T);
+        }
+        if (!PA) {
+            ca = __reduce_min_sync(kFull, lane < T ? wmin[lane] : kBig) + c.cap_a;
+            cb = __reduce_min_sync(kFull, lane < T ? wmin[kMaxT + lane] : kBig) + c.cap_b;
+        }
+        {
+            using CL = std::conditional_t<R == 3, C2, C1>;
+            const Dt &dl = R == 3 ? d2 : d1;
+            const int nl = R == 3 ? n2 : n1;
+            const unsigned nb = w.to_mbox ? stn : c.xb, stl = R == 3 ? st2 : st1;
+            auto last = [&](const Seg &s, const bool vb) {
+                phase_r<CL, X, PA>(s, dl, vb ? c.xb : c.xa, vb ? nb : c.xa, stl, vb ? c.lam_b : c.lam_a, vb ? cb : ca);
+            };
+            if (wt < 2 * nl) {
+                last(s2, wt >= nl);
+#pragma unroll 1
+                for (int t = wt + T; t < 2 * nl; t += T)
+                    last(seg_of<CL>(A.seg[R - 1], A.ax[R - 1], (t >= nl ? t - nl : t) * CL::lpw, lane), t >= nl);
+            }
+        }
+        if (__builtin_expect(stop != 0, 0)) break;
+        __syncwarp();
+        mbar_arrive_if(lane == 0, bars + kOutB + par);
+        mbar_arrive_if(lane == 0 && w.to_mbox, nx_ready + sto);
+        team_sync(tm, T);
+        par ^= 8;
+        c.ma = c.xa;
+        c.xa = xa_sum - c.xa;
+        c.xb = xb_sum - c.xb;
+        csh = (csh + dcs) & 3;
+        sto += 8;
+        const bool wrap = sto == send;
+        sta = wrap ? st0 : sta + stb;
+        stn = wrap ? nx : stn + stb;
+        sph ^= wrap ? 1u : 0u;
+        sto = wrap ? 0u : sto;
+    }
 }
 
 }  // namespace line2
 
-// One row band of one scan pass (or paired sweep) for a label space of
-// LB x LA labels (axis 0: LB labels, contiguous; axis 1: LA labels), lines
-// split over lane pairs.  Every thread of the block calls it with the same
-// band; returns false when the pass was aborted (a wait timed out).
-template <int LA, int LB, int CH, bool FUSED>
-__device__ __forceinline__ bool line2_band(const TeamArgs &A, const int band, int *smem, volatile int *s_abort) {
-    using namespace line;
-    using line2::kPQ;
-    static_assert(LA >= 33 && LA <= 65 && LB >= 33 && LB <= 65, "lines of 33 to 65 labels");
-    constexpr int NA = LA - 32 > 32 ? LA - 32 : 32;  // register line of phase A
-    constexpr int NBr = LB - 32 > 32 ? LB - 32 : 32;  // and of phase B
-    constexpr int XS = line2::buf_ints(LA);
-    constexpr size_t TI = line2::team_ints(LA);
-    constexpr int KC = line2::kCtl;
-    const int W = A.W, H = A.H, Q = A.Q, Qm = A.Qm, TW = A.T, NT = A.NT, ring = A.ring;
+// One work item: half h of the launch's sweep over the rows of one band.
+// Every thread of the block calls it; returns false when the pass was
+// aborted (a wait timed out).
+template <class B, bool FUSED>
+__device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const int band, int *smem,
+                                           volatile int *s_abort) {
+    using namespace line2;
+    const int W = A.W, H = A.H, Q = A.Q, Qm = A.Qm, T = A.T, NT = A.NT;
+    const int nst = A.nbuf, ring = A.ring;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tm = warp / TW, wt = warp - tm * TW, tl = wt * 32 + lane;
-    const int hf = lane >> 4, j = wt * 16 + (lane & 15);  // half, line
-    const bool lo = hf == 0;
-    for (int i = tid; i < NT * KC; i += blockDim.x) smem[(size_t)(i / KC) * TI + i % KC] = 0;
+    const bool copy = warp >= NT * T;
+    const int tm = copy ? (warp - NT * T) / kCopyWarps : warp / T;
+    const int wt = copy ? (warp - NT * T) % kCopyWarps : warp - tm * T;  // role / compute warp of the team
+    // shared memory: a zero vector, then the teams (stages, X_a, X_b, control)
+    const size_t TI = team_ints(Qm, nst, B::extra);
+    int *const zero = smem;
+    auto team_of = [&](int i) { return smem + Qm + (size_t)i * TI; };
+    auto ctl_of = [&](int i) { return team_of(i + 1) - kCtlInts; };
+    int *const tb = team_of(tm);
+    int *const XA = tb + nst * stage_ints(Qm);
+    int *const XB = XA + 2 * (size_t)Qm;
+    int *const ctl = ctl_of(tm);
+    int *const wmin = ctl + 32, *const wkey = ctl + 80;
+    auto bars_of = [&](int i) { return saddr(ctl_of(i)); };
+    const unsigned bars = bars_of(tm);
+
+    for (int i = tid; i < NT * kBars; i += blockDim.x) {
+        const int t = i / kBars;
+        const unsigned o = 8u * (unsigned)(i - t * kBars);
+        const int n = o >= kEmptyB ? T                                   // the compute warps
+                      : o >= kReadyB ? 1 + (t > 0 ? T : 0)               // out, the compute warps of the team above
+                                     : 1 + (t == 0 && band > 0 ? 1 : 0); // stage, above
+        mbar_init(bars_of(t) + o, (unsigned)n);
+    }
+    for (int i = tid; i < Qm; i += blockDim.x) zero[i] = 0;
+    if (tid < NT) ctl_of(tid)[30] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
     __syncthreads();
-    const unsigned long long t_band0 = (A.trace && tid == 0) ? global_ns() : 0;
+    if (A.trace && tid == 0 && h == 0) A.trace[band * 4 + 0] = global_ns();
 
     const int r = band * NT + tm;
-    if (tm < NT && r < H) {
-        const bool incy = A.pass < 2;
-        int *const Mb = incy ? A.M[2] : A.M[3];
-        const int *const Md = incy ? A.M[3] : A.M[2];
-        const int y = incy ? r : H - 1 - r;
-        const bool has_next = r + 1 < H;
-        const bool to_mbox = has_next && tm + 1 < NT;
-        const bool to_ring = has_next && tm + 1 == NT;
-        const bool from_mbox = r > 0 && tm > 0;
-        const bool from_ring = r > 0 && tm == 0;
-        const bool d_ok = A.read_d && (incy ? y + 1 < H : y - 1 >= 0);
-        const bool per_axis = A.mode == 1;
-        int *const ctl = smem + (size_t)tm * TI;
-        int *const Xa = ctl + KC;
-        int *const nx_slots = to_mbox ? smem + (size_t)(tm + 1) * TI + KC + XS : nullptr;
-        const int *const nx_ctl = to_mbox ? smem + (size_t)(tm + 1) * TI : nullptr;
-        const int *const pv_ctl = from_mbox ? smem + (size_t)(tm - 1) * TI : nullptr;
-        // the ring of slot images between blocks: [band][ring][XS] ints; the
-        // team's thread tl moves the 16-byte chunks tl, tl + 32 TW, ...
-        int *const llv = reinterpret_cast<int *>(A.ll);
-        const int *const ll_in = from_ring ? llv + (size_t)(band - 1) * ring * XS : nullptr;
-        int *const ll_out = to_ring ? llv + (size_t)band * ring * XS : nullptr;
-        const unsigned *const flag_in = from_ring ? A.rflag + (size_t)(band - 1) * kLineFlagStride + wt : nullptr;
-        unsigned *const flag_out = to_ring ? A.rflag + (size_t)band * kLineFlagStride + wt : nullptr;
-        unsigned *const cons_in = from_ring ? A.cons + (size_t)(band - 1) * kLineFlagStride + wt : nullptr;
-        const unsigned *const cons_out = to_ring ? A.cons + (size_t)band * kLineFlagStride + wt : nullptr;
-        // the test hook hold_band makes one band wait for a column never published
-        const int hold = band == A.hold_band ? 0x20000000 : 0;
-        const int ncol = A.pair ? 2 * W : W;
-        const bool colA = j < LB, rowB = j < LA;
-        const unsigned mA = __ballot_sync(kFull, colA), mB = __ballot_sync(kFull, rowB);
-        const int nA = lo ? 32 : LA - 32, nB = lo ? 32 : LB - 32;
-        const int jj = j >= 32 ? j - 32 : j;
-        const int offA = line2::qbase(LA, hf, j >= 32) + jj;        // X(32 hf + n, j) at offA + n kPQ
-        const int offB = line2::qbase(LA, j >= 32, hf) + jj * kPQ;  // X(j, 32 hf + n) at offB + n
-        const int q0 = hf * 32 * LB + j;                             // label of the lane's first phase-A entry
-        unsigned cons_seen = 0;
-        for (int s = 0; s < ncol; ++s) {
-            const int hh = s >= W ? 1 : 0;
-            const int xs = s - hh * W;
-            const bool incx = ((A.pass + hh) & 1) == 0;
-            const bool fin = hh ? A.final2 : A.final_;
-            const bool read_c = hh ? A.read_c2 : A.read_c;
-            const bool write_a = hh ? A.write_a2 : A.write_a;
-            const bool write_b = hh ? A.write_b2 : A.write_b;
-            int *const Ma = incx ? A.M[0] : A.M[1];
-            const int *const Mc = incx ? A.M[1] : A.M[0];
-            const int x = incx ? xs : W - 1 - xs;
-            const size_t pix = (size_t)y * W + x;
-            const bool has_ma = xs > 0, nxt = xs + 1 < W;
-            const bool c_ok = read_c && (incx ? x + 1 < W : x - 1 >= 0);
-            int *const Xb = Xa + (1 + (s & 1)) * XS;
-            if (s + 1 < ncol) {  // L2 prefetch of the next column's C, m_c, m_d
-                const int s2 = s + 1, h2 = s2 >= W ? 1 : 0, xs2 = s2 - h2 * W;
-                const bool incx2 = ((A.pass + h2) & 1) == 0;
-                const int x2 = incx2 ? xs2 : W - 1 - xs2;
-                const size_t p2 = (size_t)y * W + x2;
-                const bool rc2 = (h2 ? A.read_c2 : A.read_c) && (incx2 ? x2 + 1 < W : x2 - 1 >= 0);
-                const int *const pc = FUSED ? nullptr : A.C + p2 * Q;
-                const int *const pm = (incx2 ? A.M[1] : A.M[0]) + p2 * Qm;
-                const int *const pd = Md + p2 * Qm;
-                for (int o = tl * 32; o < Q; o += 32 * 32 * TW) {
-                    if (!FUSED) prefetch_line_l2(pc + o);
-                    if (rc2) prefetch_line_l2(pm + o);
-                    if (d_ok) prefetch_line_l2(pd + o);
-                }
-            }
-            int lam_a = A.lam, lam_b = A.lam, cap_a = A.capv, cap_b = A.capv;
-            if (A.wh) {
-                const int wa = nxt ? __ldg(A.wh + (size_t)y * W + (incx ? x : x - 1)) : 1;
-                const int wb = has_next ? __ldg(A.wv + (size_t)(incy ? y : y - 1) * W + x) : 1;
-                lam_a *= wa;
-                cap_a *= wa;
-                lam_b *= wb;
-                cap_b *= wb;
-            }
+    const bool row_on = r < H;
+    const bool incx = ((A.pass + h) & 1) == 0, incy = A.pass < 2;
+    const bool read_c = h ? A.read_c2 : A.read_c, write_a = h ? A.write_a2 : A.write_a;
+    const bool write_b = h ? A.write_b2 : A.write_b, fin = h ? A.final2 : A.final_;
+    const int y = incy ? r : H - 1 - r;
+    const bool has_next = r + 1 < H;
+    const bool to_mbox = has_next && tm + 1 < NT, to_ring = has_next && tm + 1 == NT;
+    const bool from_ring = r > 0 && tm == 0;
+    const bool d_ok = A.read_d && (incy ? y + 1 < H : y - 1 >= 0);
+    int *const Ma = incx ? A.M[0] : A.M[1];
+    const int *const Mc = incx ? A.M[1] : A.M[0];
+    int *const Mb = incy ? A.M[2] : A.M[3];
+    const int *const Md = incy ? A.M[3] : A.M[2];
+    int *const ringv = reinterpret_cast<int *>(A.ll);  // [band][ring][Qm]
+    const int col0 = h * W;                              // column counters run on over both halves
+    const unsigned vbytes = 4u * (unsigned)Qm;
+    const unsigned stb = 4u * (unsigned)stage_ints(Qm);  // bytes of a stage
+    const unsigned omc = vbytes + 16, omd = 2 * vbytes + 16, omb = 3 * vbytes + 16;  // m_c, m_d, m_b in it
+    const long long lim = A.spin_limit;
 
-            // ---- waits (each warp for itself; warp-uniform outcomes) ----
-            bool bad = false;
-            long long spins = 0;
-            if (from_mbox) {  // m_b of column s from every warp of the team above
-                while (true) {
-                    const bool ok = lane >= TW || ld_acq_cta(pv_ctl + lane) >= s + 1;
-                    if (__all_sync(kFull, ok)) break;
-                    if (__any_sync(kFull, ++spins > A.spin_limit || *s_abort != 0)) {
-                        bad = true;
-                        break;
+    if (copy && lane == 0 && wt < 2) ctl[28 + wt] = 0;
+    if (copy && row_on && lane == 0) {
+        int si = 0;       // stage of the column
+        unsigned ph = 0;  // its phase
+        bool ok = true;
+        auto advance = [&](int by) {
+            si += by;
+            while (si >= nst) {
+                si -= nst;
+                ph ^= 1;
+            }
+        };
+        if (wt == 0) {
+            // ---- stage: C, m_c, m_d of every column ----
+            if (h == 1) {  // this row of the first half is complete (both its out warps)
+                ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status);
+                fence_async();
+            }
+            const size_t NQ = (size_t)W * H * Q;
+            for (int xs = 0; xs < W && ok; ++xs, advance(1)) {
+                if (xs >= nst && !(ok = mbar_wait(bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort))) break;
+                const size_t pix = (size_t)y * W + (incx ? xs : W - 1 - xs);
+                const bool c_ok = read_c && xs + 1 < W;
+                const unsigned dst = saddr(tb) + (unsigned)si * stb, bar = bars + kLoadB + 8 * si;
+                unsigned cbytes = 0;
+                size_t a0 = 0;
+                if (!FUSED) {
+                    // whole 16-byte chunks around the pixel's labels; the array's
+                    // last labels, short of a chunk, by plain loads
+                    const size_t e0 = pix * Q, e1 = e0 + Q;
+                    a0 = e0 & ~(size_t)3;
+                    size_t a1 = (e1 + 3) & ~(size_t)3;
+                    if (a1 > NQ) {
+                        a1 = max(e1 & ~(size_t)3, a0);
+                        for (size_t e = a1; e < e1; ++e) tb[(size_t)si * stage_ints(Qm) + (e - a0)] = A.C[e];
                     }
+                    cbytes = 4u * (unsigned)(a1 - a0);
                 }
-                __syncwarp();
-            } else if (from_ring) {
-                // the producing warp's chunks of column s: published flag
-                // (acquired by every lane, which orders its copies after it)
-                while (true) {
-                    const bool ok = (int)line2::ld_acq_gpu(flag_in) >= s + 1 + hold;
-                    if (__all_sync(kFull, ok)) break;
-                    if (__any_sync(kFull, ++spins > A.spin_limit || *s_abort != 0 ||
-                                              ((spins & 63) == 0 && *(volatile int *)A.status != 0))) {
-                        bad = true;
-                        break;
+                mbar_arrive_tx(bar, cbytes + (c_ok ? vbytes : 0) + (d_ok ? vbytes : 0));
+                if (cbytes) bulk_load(dst, A.C + a0, cbytes, bar);
+                if (c_ok) bulk_load(dst + omc, Mc + pix * Qm, vbytes, bar);
+                if (d_ok) bulk_load(dst + omd, Md + pix * Qm, vbytes, bar);
+                ctl[28] = xs + 1;
+            }
+        } else if (wt == 1) {
+            // ---- above: m_b of every column the previous band published ----
+            if (from_ring) {
+                const unsigned *const flag = A.rflag + (size_t)(band - 1) * kLineFlagStride;
+                unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride;
+                // the test hook hold_band makes one band wait for a column never published
+                const int hold = band == A.hold_band ? 0x20000000 : 0;
+                int seen[2] = {0, 0};  // published columns as last read, even / odd
+                for (int xs = 0; xs < W && ok; ++xs, advance(1)) {
+                    const int s = col0 + xs;
+                    if (xs >= nst) {
+                        if (!(ok = mbar_wait(bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort))) break;
+                        // column s - nst has left the ring (the compute warps have
+                        // read it from shared memory)
+                        st_relaxed_gpu(cons, (unsigned)(s - nst + 1));
                     }
-                    __nanosleep(32);
-                }
-                if (!bad) {
-                    const int *const src = ll_in + (size_t)(s % ring) * XS;
-                    for (int c = tl; c < XS / 4; c += 32 * TW) line2::cp_async16(Xb + 4 * c, src + 4 * c);
-                    line2::cp_async_wait_all();
-                    // the chunks are in shared memory: the producer may reuse them
-                    __syncwarp();
-                    if (lane == 0) st_relaxed_gpu(cons_in, (unsigned)(s + 1));
-                }
-                team_sync(tm, TW);  // every warp's chunks of the slot have arrived
-            }
-            if (!bad && to_mbox) {  // the slot of this column in the team below is free
-                spins = 0;
-                while (true) {
-                    const bool ok = lane >= TW || ld_acq_cta(nx_ctl + 8 + lane) >= s - 1;
-                    if (__all_sync(kFull, ok)) break;
-                    if (__any_sync(kFull, ++spins > A.spin_limit || *s_abort != 0)) {
-                        bad = true;
-                        break;
+                    for (long long n = 0; (s & 1 ? seen[1] : seen[0]) < s + 1 + hold; ++n) {
+                        if (n > lim || *s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint2 v = ld_acq_gpu2(flag);
+                        seen[0] = (int)v.x;
+                        seen[1] = (int)v.y;
                     }
+                    if (!ok) break;
+                    fence_async();
+                    const int *const src = write_b ? Mb + ((size_t)y * W + (incx ? xs : W - 1 - xs)) * Qm
+                                                   : ringv + ((size_t)(band - 1) * ring + s % ring) * Qm;
+                    const unsigned bar = bars + kLoadB + 8 * si;
+                    mbar_arrive_tx(bar, vbytes);
+                    bulk_load(saddr(tb) + (unsigned)si * stb + omb, src, vbytes, bar);
+                    ctl[29] = xs + 1;
                 }
+                for (int xs = max(0, W - nst); xs < W && ok; ++xs)
+                    ok = mbar_wait(bars + kEmptyB + 8 * (xs % nst), (xs / nst) & 1, lim, s_abort);
+                if (ok) st_relaxed_gpu(cons, (unsigned)(col0 + W));
             }
-
-            // ---- phase A: sums of Eq. DP_2D_base, halving, sweeps along axis 1 ----
-            unsigned long long key = ~0ull;
-            int lmin_a = kBig, lmin_b = kBig;
-            int hv[NA];
-            if (!bad && colA) {
-                const bool st_a = write_a && has_ma, st_b = write_b && r > 0;
-                line2::FusedCost fc{};
-                if constexpr (FUSED) {
-                    const int xs = x + A.fv0 + A.ft0 * j;
-                    fc.col_ok = (unsigned)xs < (unsigned)W;
-                    fc.col = A.fI1 + (fc.col_ok ? xs : 0);
-                    fc.ys0 = y + A.fv1 + A.ft1 * 32 * hf;
-                    fc.t1 = A.ft1;
-                    fc.H = H;
-                    fc.pitch = A.fpitch;
-                    fc.i0 = A.fI0[(size_t)y * A.fpitch + x];
-                    fc.cmax = A.fcmax;
-                    fc.l2 = A.fl2;
-                }
-                line2::half_load<NA, LB, CH, FUSED>(FUSED ? nullptr : A.C + pix * Q + q0, fc, Mc + pix * Qm + q0,
-                                                    Md + pix * Qm + q0,
-                                             Ma + pix * Qm + q0, Mb + pix * Qm + q0, Xa + offA, Xb + offA, c_ok,
-                                             d_ok, has_ma, r > 0, st_a, st_b, fin, nA, q0, hv, lmin_a, lmin_b,
-                                             key);
-                const int la = min(lmin_a, __shfl_xor_sync(mA, lmin_a, 16));
-                const int lb = min(lmin_b, __shfl_xor_sync(mA, lmin_b, 16));
-                line2::split_sweeps<NA>(hv, lo, lam_a, per_axis ? la + cap_a : kBig, mA);
-#pragma unroll
-                for (int i = 0; i < NA; ++i)
-                    if (i < nA) Xa[offA + i * kPQ] = hv[i];
-#pragma unroll
-                for (int i = 0; i < NA; ++i) hv[i] = i < nA ? Xb[offA + i * kPQ] : kBig;
-                line2::split_sweeps<NA>(hv, lo, lam_b, per_axis ? lb + cap_b : kBig, mA);
-#pragma unroll
-                for (int i = 0; i < NA; ++i)
-                    if (i < nA) Xb[offA + i * kPQ] = hv[i];
-            }
-            if (!per_axis) {
-                const int ja = __reduce_min_sync(kFull, lmin_a), jb = __reduce_min_sync(kFull, lmin_b);
-                if (lane == 0) {
-                    ctl[16 + wt] = ja;
-                    ctl[24 + wt] = jb;
-                }
-            }
-            if (fin) {
-                key = warp_min_key(key);
-                if (lane == 0) reinterpret_cast<unsigned long long *>(ctl + 32)[wt] = key;
-            }
-            if (bad) {
-                atomicCAS(A.status, 0, EDP_ERR_TIMEOUT_CODE);
-                *s_abort = 1;
-            }
-            if (team_sync_or(tm, TW, bad || *s_abort != 0)) break;  // barrier: phase A done
-            if (fin && tl == 0) {
-                unsigned long long best = reinterpret_cast<unsigned long long *>(ctl + 32)[0];
-                for (int w = 1; w < TW; ++w) best = min(best, reinterpret_cast<unsigned long long *>(ctl + 32)[w]);
-                A.labels[pix] = (int)(best & 0xffffffffu);
-            }
-
-            // ---- phase B: sweeps along axis 0, clip, outputs ----
-            if (rowB) {
-                int ga = kBig, gb = kBig;
-                if (!per_axis)
-                    for (int w = 0; w < TW; ++w) {
-                        ga = min(ga, ctl[16 + w]);
-                        gb = min(gb, ctl[24 + w]);
-                    }
-                int *const ra = Xa + offB;
-                int *const rb = Xb + offB;
-                int gv[NBr];
-                int lm = kBig;
-#pragma unroll
-                for (int i = 0; i < NBr; ++i) {
-                    gv[i] = i < nB ? ra[i] : kBig;
-                    lm = min(lm, gv[i]);
-                }
-                lm = min(lm, __shfl_xor_sync(mB, lm, 16));
-                line2::split_sweeps<NBr>(gv, lo, lam_a, (per_axis ? lm : ga) + cap_a, mB);
-                if (nxt) {  // m_a of the next column of the row
-#pragma unroll
-                    for (int i = 0; i < NBr; ++i)
-                        if (i < nB) ra[i] = gv[i];
-                }
-                lm = kBig;
-#pragma unroll
-                for (int i = 0; i < NBr; ++i) {
-                    gv[i] = i < nB ? rb[i] : kBig;
-                    lm = min(lm, gv[i]);
-                }
-                lm = min(lm, __shfl_xor_sync(mB, lm, 16));
-                line2::split_sweeps<NBr>(gv, lo, lam_b, (per_axis ? lm : gb) + cap_b, mB);
-                if (to_mbox) {  // m_b of this column of the row below
-                    int *const nb = nx_slots + (s & 1) * XS + offB;
-#pragma unroll
-                    for (int i = 0; i < NBr; ++i)
-                        if (i < nB) nb[i] = gv[i];
+        } else {
+            // ---- out p: the finished columns p, p + 2, ... ----
+            const int p = wt - 2;
+            const unsigned *const cons = A.cons + (size_t)band * kLineFlagStride;
+            unsigned *const flag = A.rflag + (size_t)band * kLineFlagStride;
+            const int y_next = incy ? y + 1 : y - 1;
+            const unsigned nx_bars = to_mbox ? bars_of(tm + 1) : 0;
+            unsigned oph = 0;
+            // the output buffers of column p are free
+            advance(p);
+            if (p < W) mbar_arrive(bars + kReadyB + 8 * si);
+            for (int xs = p; xs < W && ok; xs += 2) {
+                const int s = col0 + xs;
+                if (!(ok = mbar_wait(bars + kOutB + 8 * p, oph, lim, s_abort))) break;
+                oph ^= 1;
+                // the compute warps' shared-memory writes (ordered by the barrier
+                // above) before the bulk copies' reads
+                fence_async();
+                const int x = incx ? xs : W - 1 - xs;
+                if (write_a && xs + 1 < W)
+                    bulk_store(Ma + ((size_t)y * W + (incx ? x + 1 : x - 1)) * Qm, saddr(XA + (size_t)(p ^ 1) * Qm), vbytes);
+                const unsigned src = to_mbox ? saddr(team_of(tm + 1)) + (unsigned)si * stb + omb
+                                             : saddr(XB + (size_t)p * Qm);
+                if (has_next && write_b) {
+                    bulk_store(Mb + ((size_t)y_next * W + x) * Qm, src, vbytes);
                 } else if (to_ring) {
-#pragma unroll
-                    for (int i = 0; i < NBr; ++i)
-                        if (i < nB) rb[i] = gv[i];
+                    if (!(ok = wait_count(cons, s - ring + 1, lim, s_abort, A.status))) break;
+                    fence_async();
+                    bulk_store(ringv + ((size_t)band * ring + s % ring) * Qm, src, vbytes);
                 }
-            }
-            if (to_mbox) {
-                __syncwarp();
-                if (lane == 0) st_rel_cta(ctl + wt, s + 1);
-            }
-            team_sync(tm, TW);  // barrier: rows of X_a (and of the outgoing slot) written
-
-            // ---- phase C (last row of the block): the outgoing slot into the ring ----
-            if (to_ring) {
-                spins = 0;
-                const int need = s - ring + 1;
-                while ((int)cons_seen < need) {
-                    cons_seen = __shfl_sync(kFull, lane == 0 ? ld_relaxed_gpu(cons_out) : 0u, 0);
-                    if ((int)cons_seen >= need) break;
-                    if (__any_sync(kFull, ++spins > A.spin_limit || *s_abort != 0 ||
-                                              ((spins & 63) == 0 && *(volatile int *)A.status != 0))) {
-                        bad = true;
+                bulk_commit();
+                bulk_wait_read();
+                advance(2);
+                if (xs + 2 < W) {
+                    // the buffers of column xs + 2 are free: those of column xs have
+                    // been read, and so has the stage of the row below
+                    if (to_mbox && xs + 2 >= nst &&
+                        !(ok = mbar_wait(nx_bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort)))
                         break;
-                    }
-                    __nanosleep(32);
+                    mbar_arrive(bars + kReadyB + 8 * si);
                 }
-                if (!bad) {
-                    int *const dst = ll_out + (size_t)(s % ring) * XS;
-                    for (int c = tl; c < XS / 4; c += 32 * TW)
-                        __stcg(reinterpret_cast<int4 *>(dst) + c, reinterpret_cast<const int4 *>(Xb)[c]);
-                }
-                // publish column s: the warp's stores, then the flag (release at
-                // GPU scope, cumulative over the stores the barrier ordered)
-                __syncwarp();
-                if (!bad && lane == 0) line2::st_rel_gpu(flag_out, (unsigned)(s + 1));
-                if (bad) {
-                    atomicCAS(A.status, 0, EDP_ERR_TIMEOUT_CODE);
-                    *s_abort = 1;
+                if (to_ring) {
+                    bulk_wait_all();
+                    fence_async();
+                    st_rel_gpu(flag + (s & 1), (unsigned)(s + 1));
                 }
             }
-            if (from_mbox) {  // this column's slot is free again for the team above
-                __syncwarp();
-                if (lane == 0) st_rel_cta(ctl + 8 + wt, s + 1);
+            bulk_wait_all();
+            if (ok && A.pair && h == 0) {
+                fence_async();
+                add_rel_gpu(A.rflag + (size_t)r * kLineFlagStride + 2, 1u);
             }
         }
+        if (!ok) timed_out(A.status, s_abort);
+    } else if (!copy && row_on) {
+        const Row w{r, y, tm, wt, lane, incx, incy, has_next, to_mbox, read_c, d_ok};
+        auto run = [&](auto fin_c, auto pa_c) {
+            B::template row<decltype(fin_c)::value, decltype(pa_c)::value, FUSED>(
+                A, w, saddr(zero), saddr(tb), saddr(XA), saddr(XB), bars, to_mbox ? saddr(team_of(tm + 1)) + omb : 0u,
+                to_mbox ? bars_of(tm + 1) + kReadyB : 0u, wmin, wkey, ctl + 30, s_abort);
+        };
+        if (A.mode == 1)
+            fin ? run(std::true_type(), std::true_type()) : run(std::false_type(), std::true_type());
+        else
+            fin ? run(std::true_type(), std::false_type()) : run(std::false_type(), std::false_type());
+    }
+    __syncthreads();
+    const bool done = *s_abort == 0;
+    if (!done && tid < NT) {
+        // an aborted item: wait (bounded) for the copies in flight into the
+        // stages; where only one of `stage` and `above` announced a column,
+        // make up the other's arrival
+        const int *const issued = ctl_of(tid) + 28;
+        const bool two = tid == 0 && band > 0;
+        const int n = max(issued[0], issued[1]);
+        if (two)
+            for (int xs = min(issued[0], issued[1]); xs < n; ++xs) mbar_arrive(bars_of(tid) + kLoadB + 8 * (xs % nst));
+        for (int xs = max(0, n - nst); xs < n; ++xs)
+            for (int k = 0; k < 1000000 && !mbar_try(bars_of(tid) + kLoadB + 8 * (xs % nst), (xs / nst) & 1); ++k) {
+            }
     }
     if (A.trace && tid == 0) {
-        A.trace[band * 4 + 0] = t_band0;
         A.trace[band * 4 + 1] = global_ns();
         A.trace[band * 4 + 2] = 0;
         A.trace[band * 4 + 3] = sm_id();
     }
     __syncthreads();
-    return *s_abort == 0;
+    for (int i = tid; i < NT * kBars; i += blockDim.x) mbar_inval(bars_of(i / kBars) + 8 * (i % kBars));
+    __syncthreads();
+    return done;
 }
 
 }  // namespace edp
