@@ -354,12 +354,13 @@ bool line2_cut(const Geometry &g, const edp_params *p, int b, Line2Shape *S) {
     if ((B.S[2] > 0 ? 3 : 2) != g.R) return false;
     for (int r = 0; r < g.R; ++r) {
         const int L = g.Qr[r], s = B.S[r], e = (L + s - 1) / s;
-        if (L < s || e > B.E[r] || (B.exact && e != B.E[r])) return false;
+        if (B.Q[0] ? L != B.Q[r] : (L < s || e > B.E[r])) return false;
         S->E[r] = e;
-        S->seg[r].S = s;
-        S->seg[r].lpw = 32 / s;
-        S->seg[r].nf = L - s * (e - 1);
-        S->seg[r].kc = std::min(s - 1, (p->g - 1 + L / s - 1) / (L / s));
+        S->seg[r].S = (short)s;
+        S->seg[r].lpw = (short)(32 / s);
+        S->seg[r].nf = (short)(L - s * (e - 1));
+        S->seg[r].kc = (short)std::min<long long>(s - 1, (p->g - 1LL + L / s - 1) / (L / s));
+        S->seg[r].near = S->seg[r].kc <= 1 && p->g <= 4;
     }
     S->build = b;
     return true;
@@ -379,10 +380,11 @@ bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, i
             double ins[3] = {0, 0, 0}, busy[3] = {0, 0, 0};  // instructions of a warp, warps at work, per phase
             int most = 1;
             for (int r = 0; r < g.R; ++r) {
-                const int lpw = S.seg[r].lpw, n = (r == 0 ? 1 : 2) * ((g.Q / g.Qr[r] + lpw - 1) / lpw);
+                const int lpw = S.seg[r].lpw, nv = r > 0 && !B.both ? 2 : 1;
+                const int n = nv * ((g.Q / g.Qr[r] + lpw - 1) / lpw);
                 const int rounds = (n + T - 1) / T;
                 most = std::max(most, n);
-                ins[r] = rounds * ((r == 0 ? 24.0 : 11.0) * B.E[r] * (B.exact ? 1.0 : 1.3) + 45.0);
+                ins[r] = rounds * ((r == 0 ? 22.0 : B.both ? 17.0 : 9.0) * B.E[r] * (B.Q[0] ? 1.0 : 1.4) + 45.0);
                 busy[r] = (double)n / rounds;
             }
             if (warps <= 0 && T > most) break;
@@ -413,6 +415,14 @@ bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, i
     }
     return have;
 }
+// Columns of the hand-off ring of the split line kernel's frame: some slack
+// when every band is resident, otherwise the depth that lets the first resident
+// band finish its row; with copies the consumer counts a column nst columns late.
+// (The workspace has room for team_ring(2W, kResidentMin) columns of records,
+// twice as many of plain values.)
+int line2_ring(bool rec, int nst, int W, int nbands, int resident) {
+    return (rec ? 0 : nst) + (nbands <= resident ? 8 : team_ring(W, std::max(1, resident)));
+}
 bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry &g, const edp_params *p,
                 int32_t *labels, unsigned char *ws, int sms, SolvePlan *P) {
     // lambda 255 (the heaviest per-edge multiplier) within the sweeps' range;
@@ -441,16 +451,14 @@ bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry 
     a.NT = S.NT;
     a.nbuf = S.nst;
     a.nbands = (H + S.NT - 1) / S.NT;
-    // hand-off ring (plain values, 4 bytes a label; the consumer counts a
-    // column nst columns late): 8 columns of slack when every band is resident,
-    // otherwise the depth that lets the first resident band finish its row
     P->nbands = a.nbands;
     P->build = S.build;
     P->threads = pass_line2_threads(S.NT, S.T);
     P->smem = pass_line2_smem(S.NT, L.Qm, S.nst);
     const int occ = edp_pass_line2_occupancy(P->build, P->threads, P->smem);
-    const int need = S.nst + (a.nbands <= occ * sms ? 8 : team_ring(W, std::max(1, occ * sms)));
-    a.ring = std::min(need, 2 * team_ring(2 * W, kResidentMin));
+    a.rec = g.Q <= pass_line2_max_rec_labels();
+    const int need = line2_ring(a.rec, S.nst, W, a.nbands, occ * sms);
+    a.ring = std::min(need, (a.rec ? 1 : 2) * team_ring(2 * W, kResidentMin));
     if (occ < 1 || a.ring < need) {  // (cannot happen with the SMs the workspace was sized for)
         memset(&P->ta, 0, sizeof P->ta);
         P->line = P->split = false;
@@ -687,7 +695,8 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
 // Control words that must start from zero before the first pass: status,
 // consumed-column and band counters, and the used hand-off records.
 size_t control_bytes(const SolvePlan &P, int W, int Q) {
-    if (P.split) return P.L.ll;  // plain values, published by the flags
+    // plain values are published by the flags; records start without a tag
+    if (P.split) return P.L.ll + (P.ta.rec ? (size_t)P.nbands * P.ta.ring * P.L.Qm * 8 : 0);
     return P.r1 ? P.L.ll + (size_t)P.nbands * 2 * W * Q * 8 : P.L.ll + (size_t)P.nbands * P.ta.ring * P.L.Qm * 8;
 }
 
@@ -808,6 +817,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
                 const int slot = it * 4 + set_launch(a, it, k, p->iters, pairs);
                 a.cons = reinterpret_cast<unsigned *>(ws + P.L.lcons) + (size_t)slot * H * kLineFlagStride;
                 a.rflag = reinterpret_cast<unsigned *>(ws + P.L.lflag) + (size_t)slot * H * kLineFlagStride;
+                a.tag0 = 1 + slot * W;  // a pair takes the tags of both its passes' slots
                 a.hold_band = g_hold_band;
                 a.band_counter = reinterpret_cast<unsigned *>(ws + P.L.counters) + slot;
                 a.grid = std::min(grid_t, P.nbands * (pairs ? 2 : 1));
@@ -1587,17 +1597,18 @@ int run_windowed(TeamArgs a, const SolveLayout &L, unsigned char *w, int iters, 
     // rows per block (a compute and four copy warps each): enough blocks for the
     // SMs first, then few hand-offs between blocks
     int NT = g_tune_rb > 0 ? g_tune_rb : std::max(1, (H + sms - 1) / sms);
-    NT = std::max(1, std::min(std::min(NT, 5), H));
+    NT = std::max(1, std::min(std::min(NT, 4), H));
     a.NT = NT;
     const int threads = pass_line2_threads(NT, 1);
     const size_t smem = pass_win_smem(NT, L.Qm, a.nbuf);
     if (smem > (size_t)kMaxSmem) return EDP_ERR_UNSUPPORTED;
     const int occ = edp_pass_win_occupancy(a.win, threads, smem);
     a.nbands = (H + NT - 1) / NT;
-    a.ring = a.nbuf + (a.nbands <= occ * sms ? 8 : team_ring(W, std::max(1, occ * sms)));
-    if (occ < 1 || a.ring > 2 * team_ring(2 * W, kResidentMin)) return EDP_ERR_UNSUPPORTED;
+    a.rec = 1;
+    a.ring = line2_ring(true, a.nbuf, W, a.nbands, occ * sms);
+    if (occ < 1 || a.ring > team_ring(2 * W, kResidentMin)) return EDP_ERR_UNSUPPORTED;
     int rc;
-    if ((rc = cuda_status(cudaMemsetAsync(w, 0, L.ll, st)))) return rc;
+    if ((rc = cuda_status(cudaMemsetAsync(w, 0, L.ll + (size_t)a.nbands * a.ring * L.Qm * 8, st)))) return rc;
     const bool pairs = pairs_for(a.nbands <= 4 * occ * sms);
     const int per_it = pairs ? 2 : 4;
     a.grid = std::min(a.nbands * (pairs ? 2 : 1), occ * sms);
@@ -1610,6 +1621,7 @@ int run_windowed(TeamArgs a, const SolveLayout &L, unsigned char *w, int iters, 
             const int slot = it * 4 + set_launch(b, it, k, iters, pairs);
             b.cons = reinterpret_cast<unsigned *>(w + L.lcons) + (size_t)slot * H * kLineFlagStride;
             b.rflag = reinterpret_cast<unsigned *>(w + L.lflag) + (size_t)slot * H * kLineFlagStride;
+            b.tag0 = 1 + slot * W;
             b.band_counter = reinterpret_cast<unsigned *>(w + L.counters) + slot;
             const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
             if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)

@@ -7,36 +7,36 @@
 namespace edp {
 
 static const Line2Build kBuilds[] = {
-    // exact cuts (segments, labels per lane of each axis): the repository's
-    // label spaces -- 65 x 65, 33 x 33, 27 x 15, 25 x 25, 17 x 17, 9 x 9,
-    // 17 x 17 x 9, 9 x 9 x 9
-    {{8, 8, 0}, {9, 9, 0}, true, 672, line2_k0},
-    {{8, 4, 0}, {5, 9, 0}, true, line2::kMaxThreads, line2_k1},
-    {{8, 4, 0}, {4, 4, 0}, true, line2::kMaxThreads, line2_k2},
-    {{8, 4, 0}, {4, 7, 0}, true, line2::kMaxThreads, line2_k3},
-    {{8, 4, 0}, {3, 5, 0}, true, line2::kMaxThreads, line2_k4},
-    {{4, 4, 0}, {3, 3, 0}, true, line2::kMaxThreads, line2_k5},
-    {{4, 2, 1}, {5, 9, 9}, true, line2::kMaxThreads, line2_k6},
-    {{4, 2, 2}, {3, 5, 5}, true, line2::kMaxThreads, line2_k7},
+    // the label spaces of the repository's workloads and tests
+    {{65, 65, 1}, {5, 5, 0}, {13, 13, 0}, true, 480, line2_k0},
+    {{33, 33, 1}, {3, 3, 0}, {11, 11, 0}, true, 512, line2_k1},
+    {{27, 15, 1}, {3, 3, 0}, {9, 5, 0}, true, 512, line2_k2},
+    {{25, 25, 1}, {3, 3, 0}, {9, 9, 0}, true, 512, line2_k3},
+    {{17, 17, 1}, {1, 1, 0}, {17, 17, 0}, true, 512, line2_k4},
+    {{9, 9, 1}, {3, 3, 0}, {3, 3, 0}, true, 640, line2_k5},
+    {{17, 17, 9}, {1, 1, 1}, {17, 17, 9}, true, 384, line2_k6},
+    {{9, 9, 9}, {1, 1, 1}, {9, 9, 9}, true, 512, line2_k7},
     // any line lengths up to segments x labels
-    {{4, 4, 0}, {4, 4, 0}, false, line2::kMaxThreads, line2_k8},
-    {{8, 4, 0}, {4, 4, 0}, false, line2::kMaxThreads, line2_k9},
-    {{8, 4, 0}, {4, 8, 0}, false, line2::kMaxThreads, line2_k10},
-    {{8, 8, 0}, {9, 9, 0}, false, 672, line2_k11},
-    {{4, 4, 4}, {4, 4, 4}, false, line2::kMaxThreads, line2_k12},
+    {{0, 0, 0}, {2, 2, 0}, {8, 8, 0}, true, 512, line2_k8},
+    {{0, 0, 0}, {4, 2, 0}, {8, 8, 0}, true, 512, line2_k9},
+    {{0, 0, 0}, {4, 4, 0}, {8, 8, 0}, true, 512, line2_k10},
+    {{0, 0, 0}, {8, 8, 0}, {9, 9, 0}, true, 512, line2_k11},
+    {{0, 0, 0}, {2, 2, 2}, {8, 8, 8}, true, 512, line2_k12},
 };
 
 int pass_line2_max_lambda() { return line2::kMaxLambda; }
 int pass_line2_builds() { return (int)(sizeof kBuilds / sizeof kBuilds[0]); }
 const Line2Build &pass_line2_build(int b) { return kBuilds[b]; }
+int pass_line2_max_rec_labels() { return line2::kMaxRecQ; }
 int pass_line2_max_warps() { return line2::kMaxT; }
 int pass_line2_threads(int NT, int T) { return 32 * NT * (T + line2::kCopyWarps); }
 
 size_t pass_line2_smem(int NT, int Qm, int nst) { return ((size_t)Qm + NT * line2::team_ints(Qm, nst, 0)) * 4; }
 
+// (dynamic shared memory beyond 48 KB with the static part needs the attribute)
 int edp_pass_line2_occupancy(int build, int threads, size_t smem) {
     void *k = kBuilds[build].kernel(false);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, smem);
     return occ;
@@ -45,7 +45,7 @@ int edp_pass_line2_occupancy(int build, int threads, size_t smem) {
 int launch_edp_pass_line2(const TeamArgs &a, int build, int threads, size_t smem, cudaStream_t st) {
     void *k = kBuilds[build].kernel(a.fI1 != nullptr);
     if (!k) return -1;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     void *args[] = {const_cast<TeamArgs *>(&a)};
     return cudaLaunchKernel(k, dim3(a.grid), dim3(threads), args, smem, st) == cudaSuccess ? 0 : -2;
 }

@@ -28,7 +28,7 @@ size_t pass_win_smem(int NT, int Qm, int nst) { return ((size_t)Qm + NT * line2:
 int edp_pass_win_occupancy(int n, int threads, size_t smem) {
     void *k = win_kernel_for(n);
     if (!k) return 0;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int occ = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, threads, smem);
     return occ;
@@ -37,7 +37,7 @@ int edp_pass_win_occupancy(int n, int threads, size_t smem) {
 int launch_edp_pass_win(const TeamArgs &a, int threads, size_t smem, cudaStream_t st) {
     void *k = win_kernel_for(a.win);
     if (!k) return -1;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > 32 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     void *args[] = {const_cast<TeamArgs *>(&a)};
     return cudaLaunchKernel(k, dim3(a.grid), dim3(threads), args, smem, st) == cudaSuccess ? 0 : -2;
 }

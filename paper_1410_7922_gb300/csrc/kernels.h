@@ -41,10 +41,11 @@ struct TeamAxis {
 };
 // lines cut into segments held by several lanes (pass_line2.cuh)
 struct SegAxis {
-    int S;        // segments (lanes) per line
-    int lpw;      // lines per warp, 32 / S
-    int nf;       // segments that hold E labels (the others hold E - 1)
-    int kc;       // segments of carry in the truncated sweeps
+    short S;      // segments (lanes) per line
+    short lpw;    // lines per warp, 32 / S
+    short nf;     // segments that hold E labels (the others hold E - 1)
+    short kc;     // segments of carry in the truncated sweeps
+    int near;     // one segment of carry, and g <= 4
 };
 struct TeamArgs {
     const int *C;           // [H][W][Q]
@@ -79,6 +80,7 @@ struct TeamArgs {
     // split line kernel: the pair cost of Eq. Cost_value computed from the
     // images (fI1 non-null) instead of read from C: offsets (fv0 + ft0 q0,
     // fv1 + ft1 q1), truncation fcmax, power fl2
+    int rec;                // split line kernel: hand-off between bands as records (else copies)
     const uint8_t *fI0, *fI1;
     int fpitch, fv0, fv1, ft0, ft1, fcmax, fl2;
 };
@@ -98,14 +100,16 @@ int launch_edp_pass_line(const TeamArgs &a, int Q0, int Q1, int threads, size_t 
 // NT = rows per block, nbuf stages
 int pass_line2_max_lambda();
 struct Line2Build {
+    int Q[3];                // the label space it is for (0: any whose lines fit)
     int S[3], E[3];          // segments per line and labels per lane of each axis (S = 0: no such axis)
-    bool exact;              // lines of exactly E or E - 1 labels per segment, else any that fit
+    bool both;               // both vectors per warp in the later phases
     int threads;             // bound of a block
     void *(*kernel)(bool fused);
 };
 int pass_line2_builds();
 const Line2Build &pass_line2_build(int b);
 int pass_line2_max_warps();
+int pass_line2_max_rec_labels();
 int pass_line2_threads(int NT, int T);
 size_t pass_line2_smem(int NT, int Qm, int nst);
 int edp_pass_line2_occupancy(int build, int threads, size_t smem);

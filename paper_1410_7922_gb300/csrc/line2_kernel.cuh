@@ -6,6 +6,9 @@ namespace edp {
 
 using line2::Build;
 using line2::Cut;
+using line2::Fixed2;
+using line2::Fixed3;
+using line2::NoCut;
 
 // FUSED: the pair cost computed from the images instead of read from C
 template <class B, bool FUSED>

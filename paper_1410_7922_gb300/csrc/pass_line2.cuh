@@ -32,31 +32,40 @@
 //   barrier.
 // The min search is separable, so the order of the axes changes no value.
 //
-// A line of L labels is cut into S segments (S a power of two) of e = ceil(L / S)
-// or e - 1 labels; lane k * lpw + l of a warp holds segment k of the warp's line
-// l (lpw = 32 / S lines per warp), so neighbouring lanes read neighbouring
-// lines (odd strides: distinct banks).  Per segment the forward and the
-// backward sweep (Eq. L_dec3, Eq. L_dec5) run on the lane's own labels; the
-// values at the segment's ends travel by one shuffle per direction, kc
-// segments far, and complete the labels they can still improve: a source
-// g or more labels away costs at least the clip value applied afterwards
-// (Sec. 3.1), so nothing beyond is needed.
+// A line of L labels is cut into S segments of e = ceil(L / S) or e - 1 labels;
+// lane k * lpw + l of a warp holds segment k of the warp's line l
+// (lpw = 32 / S lines per warp), so neighbouring lanes read neighbouring lines
+// (odd strides: distinct banks; 65 labels in 5 segments of 13, 33 in 3 of 11 or
+// 8 of 4-5 put all lanes on distinct banks, 65 in 8 segments would not: its
+// segments 32 labels apart share a bank).  Lanes without a line or a segment
+// repeat another one, stores included, so nothing is predicated.  Per
+// segment the forward and the backward sweep (Eq. L_dec3, Eq. L_dec5) run on the
+// lane's own labels; the values at the segment's ends travel by one shuffle per
+// direction, kc segments far, and complete the labels they can still improve:
+// a source g or more labels away costs at least the clip value applied
+// afterwards (Sec. 3.1), so nothing beyond is needed.
 //
 // A column step is a few hundred instructions in a row, run by a few warps per
 // scheduler, so what costs is not the arithmetic but every taken branch and
 // every load from the parameter block (tens of cycles each).  Hence one build
-// per cut of the axes (labels per lane as constants, EXACT where the cut
-// matches e), the truncation mode and the last pass as separate copies of the
-// column loop, and predicated single instructions instead of short branches.
-// (A build that picked the cut at run time took 2.2 us a column at 33 x 33
-// labels.)
+// per label space of the repository's workloads (all sizes constants) and a
+// few for any other (up to E labels per lane), the truncation mode and the
+// last pass as separate copies of the column loop.  (A build that picked the
+// cut at run time took 2.2 us a column at 33 x 33 labels.)
 //
-// Between bands.  The messages m_b are in global memory either way: in the
-// passes that keep them, in the message array M[b] itself; in the others in a
-// ring of `ring` columns per band that stays in L2.  The producing `out` warp
-// publishes a column when its copies have completed (release at GPU scope);
-// the `above` warp of the next band acquires it and copies it in.  A ring slot
-// is written again once the consumer has counted its column (cons).
+// Between bands, m_b goes through a ring of `ring` columns per band in global
+// memory that stays in L2, in one of two forms:
+//   records (A.rec, up to kMaxRecQ labels): the compute warps of a band's last
+//           row store {value, tag} words themselves, and the `above` warp of
+//           the next band polls them into its stage -- a matching tag carries
+//           its value, so no fence, flag or copy completion is on the path;
+//   copies  (longer vectors, twice whose bytes would load L2): the `out` warp
+//           copies X_b to the ring (or, in the passes that keep m_b, to the
+//           message array anyway) and publishes the column when the copy has
+//           completed (release at GPU scope); `above` acquires that and copies.
+// A ring slot is written again once the consumer has counted its column (cons).
+// (33 x 33 labels, 320x240: 3.7 ms a solve with copies, T = 0.9 us a column but
+// 4 us a hand-off, and at most one column a microsecond through it.)
 //
 // Work items.  A launch holds one pass, or two that share the vertical
 // direction (A.pair: P1 then P2, or P3 then P4) as items (half, band) claimed
@@ -78,6 +87,7 @@ constexpr int kCopyWarps = 4;     // stage, above, out 0, out 1
 constexpr int kMaxT = 24;         // compute warps of a team
 constexpr int kMaxThreads = 896;  // of a block: 72 registers a thread
 constexpr int kMaxStages = 4;
+constexpr int kMaxRecQ = 512;     // labels of the record form
 // control ints of one team: mbarriers [0, 28), columns issued by `stage` and
 // `above` (an aborted item's, [28, 30)), abort flag [30], warp minima [32, 80), warp argmin
 // values and labels [80, 128)
@@ -162,6 +172,16 @@ __device__ __forceinline__ uint2 ld_acq_gpu2(const unsigned *p) {
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return make_uint2((unsigned)v, (unsigned)(v >> 32));
 }
+// {value, tag} records: single 64-bit accesses (two of them in one load)
+__device__ __forceinline__ void st_rec(int2 *p, int v, int tag) {
+    const unsigned long long w = (unsigned long long)(unsigned)v | ((unsigned long long)(unsigned)tag << 32);
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ int4 ld_rec2(const int2 *p) {
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    return make_int4((int)(unsigned)a, (int)(a >> 32), (int)(unsigned)b, (int)(b >> 32));
+}
 __device__ __forceinline__ void st_relaxed_gpu(unsigned *p, unsigned v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -193,72 +213,73 @@ __device__ __forceinline__ bool team_sync_or(int tm, int T, bool pred) {
     return r != 0;
 }
 
-// predicated single instructions
-__device__ __forceinline__ void sts_if(bool p, unsigned a, int v) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %2, 0;\n\t@q st.shared.s32 [%0], %1;\n\t}" ::"r"(a), "r"(v),
-                 "r"((int)p)
-                 : "memory");
-}
+// one lane's arrival, without a branch
 __device__ __forceinline__ void mbar_arrive_if(bool p, unsigned b) {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %1, 0;\n\t@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(b),
                  "r"((int)p)
                  : "memory");
 }
 
-// The cut of one axis: S segments per line, at most E labels each.
-template <int S_, int E_>
+// The cut of one axis: S segments per line, at most E labels each.  L, LINES,
+// STRIDE: the axis' sizes where the build fixes them (L = 0: run time).
+template <int S_, int E_, int L_ = 0, int LINES_ = 0, int STRIDE_ = 0>
 struct Cut {
-    static constexpr int S = S_, E = E_, lpw = 32 / S_;
+    static constexpr int S = S_, E = E_, L = L_, lpw = 32 / S_;
+    static constexpr bool fixed = L_ > 0;
+    static constexpr bool full = L_ == S_ * E_;      // every segment holds E labels
+    static constexpr int NF = L_ - S_ * (E_ - 1);    // fixed: segments of E labels
+    static_assert(!fixed || (NF >= 1 && NF <= S_), "lines cut into segments of E or E - 1 labels");
+    static __device__ __forceinline__ int nlines(const TeamArgs &A, int r) { return fixed ? LINES_ : A.ax[r].nlines; }
+    static __device__ __forceinline__ int stride(const TeamArgs &A, int r) { return fixed ? STRIDE_ : A.ax[r].stride; }
+    static __device__ __forceinline__ int len(const TeamArgs &A, int r) { return fixed ? L_ : A.ax[r].L; }
+    // first position of segment k: the last nf segments hold e labels, the others
+    // e - 1 (33 labels in 8 segments start at 0, 4, .. 28: with 4 lines a warp,
+    // on distinct banks; the long segment first would put two on one bank)
+    static __device__ __forceinline__ int pos(const TeamArgs &A, int r, int k) {
+        const int e = fixed ? E_ : A.ax[r].E, nf = fixed ? NF : A.seg[r].nf;
+        return k * (e - 1) + max(0, k - (S - nf));
+    }
 };
 
 // A lane's place on one axis.
 struct Seg {
-    int k;             // segment
+    int k, l;          // segment, line within the warp
     int off;           // linear index of the segment's first label
     int n;             // its labels
-    int gl, gr;        // labels between the segment's position 0 and the (virtual) last one of the segment before,
-                       // and between its (virtual) last one and position 0 of the segment after
-    bool on;           // the lane serves a line
+    int sl, sr, s2;    // lanes of the segments before, after (cyclic), two after (cyclic)
 };
-// first position of segment k (the first nf segments hold e labels, the rest e - 1)
-__device__ __forceinline__ int seg_pos(int k, int e, int nf) { return k * (e - 1) + min(k, nf); }
-// the lane's place when the warp serves the lines from li0
+// the lane's place when the warp serves the lines from li0 (lines past the
+// last one, and lanes past the last segment, repeat)
 template <class C>
-__device__ __forceinline__ Seg seg_of(const SegAxis &G, const TeamAxis &X, int li0, int lane) {
+__device__ __forceinline__ Seg seg_of(const TeamArgs &A, int r, int li0, int lane) {
     Seg s;
-    s.k = lane / C::lpw;
-    const int li = li0 + lane - s.k * C::lpw;
-    s.on = li < X.nlines;
-    const int p = seg_pos(s.k, X.E, G.nf);
-    s.n = seg_pos(s.k + 1, X.E, G.nf) - p;
-    s.gl = p - seg_pos(s.k - 1, X.E, G.nf) - C::E + 1;
-    s.gr = s.n - C::E + 1;
-    s.off = 0;
-    if (s.on) {
-        // first label of line li
-        int f = li;
-        if (X.stride == 1)
-            f = li * X.L;
-        else if (li >= X.stride)
-            f = (li % X.stride) + (li / X.stride) * X.stride * X.L;
-        s.off = f + p * X.stride;
-    }
+    s.k = min(lane / C::lpw, C::S - 1);
+    s.l = lane - (lane / C::lpw) * C::lpw;
+    const int nl = C::nlines(A, r), st = C::stride(A, r), L = C::len(A, r);
+    const int li = min(li0 + s.l, nl - 1);
+    const int p = C::pos(A, r, s.k);
+    s.n = C::pos(A, r, s.k + 1) - p;
+    s.sl = max(s.k - 1, 0) * C::lpw + s.l;
+    s.sr = (s.k + 1) % C::S * C::lpw + s.l;
+    s.s2 = (s.k + 2) % C::S * C::lpw + s.l;
+    // first label of line li
+    int f = li;
+    if (st == 1)
+        f = li * L;
+    else if (li >= st)
+        f = (li % st) + (li / st) * st * L;
+    s.off = f + p * st;
     return s;
 }
 
-// The min search's constants of a pass: carries from kc segments; near: one
-// segment, and only the labels next to a boundary can improve (g <= 4).
-struct Dt {
-    int kc, e, nf;
-    bool near;
-};
-
 // Truncated L1 distance transform and clip of one vector's segment, in place
 // (positions n .. E - 1 hold kBig); cl is the clip value.  f, b: the lane's
-// own sweeps.
-template <class C, bool EXACT>
-__device__ __forceinline__ void seg_dt(int (&h)[C::E], const Seg &s, const Dt &D, const int lam, const int cl) {
-    constexpr int E = C::E;
+// own sweeps.  near: carries from one segment, and only labels next to a
+// boundary can improve (g <= 4).
+template <class C>
+__device__ __forceinline__ void seg_dt(const TeamArgs &A, const int r, int (&h)[C::E], const Seg &s, const bool near,
+                                       const int lam, const int cl) {
+    constexpr int E = C::E, S = C::S;
     int f[E], b[E];
     f[0] = h[0];
     b[E - 1] = h[E - 1];
@@ -267,21 +288,33 @@ __device__ __forceinline__ void seg_dt(int (&h)[C::E], const Seg &s, const Dt &D
         f[i] = __viaddmin_s32(f[i - 1], lam, h[i]);
         b[E - 1 - i] = __viaddmin_s32(b[E - i], lam, h[E - 1 - i]);
     }
-    if constexpr (C::S > 1) {
+    if constexpr (S > 1) {
         // carries: cf at position 0 of the segment, cb at position E - 1
         const int F = f[E - 1], B = b[0];
-        int cf = __shfl_up_sync(kFull, F, C::lpw) + lam * s.gl, cb = __shfl_down_sync(kFull, B, C::lpw) + lam * s.gr;
+        int cf = __shfl_sync(kFull, F, s.sl), cb = __shfl_sync(kFull, B, s.sr);
+        if constexpr (C::full) {
+            cf += lam;
+            cb += lam;
+        } else if constexpr (C::fixed) {
+            cf += s.k > S - C::NF ? lam : 0;
+            cb += s.k >= S - C::NF ? lam : 0;
+        } else {
+            cf += lam * (C::pos(A, r, s.k) - C::pos(A, r, s.k - 1) - E + 1);
+            cb += lam * (s.n - E + 1);
+        }
         cf = s.k > 0 ? cf : kBig;
-        cb = s.k + 1 < C::S ? cb : kBig;
+        cb = s.k < S - 1 ? cb : kBig;
         // labels within 3 of the segment's ends, or all of them
-        constexpr int NF = EXACT && E > 3 ? 3 : E, NB = EXACT && E > 4 ? 4 : E;
-        if (__builtin_expect(!D.near, 0)) {
+        constexpr int NF = C::fixed && E > 3 ? 3 : E, NB = C::full && E > 3 ? 3 : C::fixed && E > 4 ? 4 : E;
+        if (__builtin_expect(!near, 0)) {
+            const int kc = A.seg[r].kc;
 #pragma unroll 1
-            for (int d = 2; d <= D.kc; ++d) {
-                const int uf = __shfl_up_sync(kFull, F, d * C::lpw), ub = __shfl_down_sync(kFull, B, d * C::lpw);
-                const int p = seg_pos(s.k, D.e, D.nf);
-                if (s.k >= d) cf = min(cf, uf + lam * (p - seg_pos(s.k - d, D.e, D.nf) - E + 1));
-                if (s.k + d < C::S) cb = min(cb, ub + lam * (seg_pos(s.k + d, D.e, D.nf) - p - E + 1));
+            for (int d = 2; d <= kc; ++d) {
+                const int uf = __shfl_sync(kFull, F, max(s.k - d, 0) * C::lpw + s.l);
+                const int ub = __shfl_sync(kFull, B, min(s.k + d, S - 1) * C::lpw + s.l);
+                const int p = C::pos(A, r, s.k);
+                if (s.k >= d) cf = min(cf, uf + lam * (p - C::pos(A, r, s.k - d) - E + 1));
+                if (s.k + d < S) cb = min(cb, ub + lam * (C::pos(A, r, s.k + d) - p - E + 1));
             }
 #pragma unroll
             for (int i = NF; i < E; ++i) f[i] = __viaddmin_s32(cf, lam * i, f[i]);
@@ -297,11 +330,23 @@ __device__ __forceinline__ void seg_dt(int (&h)[C::E], const Seg &s, const Dt &D
     for (int i = 0; i < E; ++i) h[i] = __vimin3_s32(f[i], b[i], cl);
 }
 
-// minimum over the line (every lane of the line gets it)
+// minimum over the line (every lane of the line gets it): windows of lanes
+// that grow modulo S (the minimum is idempotent)
 template <class C>
-__device__ __forceinline__ int line_min(int m) {
+__device__ __forceinline__ int line_min(int m, const Seg &s) {
+    constexpr int S = C::S;
+    if constexpr (S == 2 || S == 4 || S == 8) {
 #pragma unroll
-    for (int d = C::lpw; d < 32; d <<= 1) m = min(m, __shfl_xor_sync(kFull, m, d));
+        for (int d = C::lpw; d < 32; d <<= 1) m = min(m, __shfl_xor_sync(kFull, m, d));
+    } else if constexpr (S == 3) {
+        m = __vimin3_s32(m, __shfl_sync(kFull, m, s.sr), __shfl_sync(kFull, m, s.s2));
+    } else if constexpr (S == 5) {
+        m = min(m, __shfl_sync(kFull, m, s.sr));    // 2 segments
+        m = min(m, __shfl_sync(kFull, m, s.s2));    // 4
+        m = min(m, __shfl_sync(kFull, m, s.sr));    // all
+    } else {
+        static_assert(S == 1, "segments per line");
+    }
     return m;
 }
 
@@ -326,8 +371,8 @@ struct In0 {
     int lam_a, lam_b, cap_a, cap_b;
     FusedPix fp;
 };
-template <class C, bool EXACT, bool FIN, bool PA, bool FUSED>
-__device__ __forceinline__ void phase0(const TeamArgs &A, const In0 &c, const Seg &s, const Dt &D, const int fq0,
+template <class C, bool FIN, bool PA, bool FUSED>
+__device__ __forceinline__ void phase0(const TeamArgs &A, const In0 &c, const Seg &s, const bool near, const int fq0,
                                        const int fq1, int &ja, int &jb, int &sv, int &sq) {
     constexpr int E = C::E;
     const unsigned o = 4u * (unsigned)s.off;
@@ -345,61 +390,108 @@ __device__ __forceinline__ void phase0(const TeamArgs &A, const In0 &c, const Se
         const int t = cv + lds(c.ma + oi) + lds(c.mb + oi);
         ha[i] = floor_half(t + md - mc);
         hb[i] = floor_half(t + mc - md);
+        const bool maybe = C::full ? false : C::fixed ? i == E - 1 : true;  // past the segment on some lanes
         if (FIN) {
             const int so = t + mc + md;
-            if (s.on && i < s.n && so < sv) {
+            if ((!maybe || i < s.n) && so < sv) {
                 sv = so;
                 sq = s.off + i;
             }
         }
-        if ((!EXACT || i == E - 1) && i >= s.n) ha[i] = hb[i] = kBig;
+        if (maybe && i >= s.n) ha[i] = hb[i] = kBig;
         ma = min(ma, ha[i]);
         mb = min(mb, hb[i]);
     }
     int ca = kBig, cb = kBig;
     if (PA) {
-        ca = line_min<C>(ma) + c.cap_a;
-        cb = line_min<C>(mb) + c.cap_b;
+        ca = line_min<C>(ma, s) + c.cap_a;
+        cb = line_min<C>(mb, s) + c.cap_b;
     } else {
-        ja = min(ja, s.on ? ma : kBig);
-        jb = min(jb, s.on ? mb : kBig);
+        ja = min(ja, ma);
+        jb = min(jb, mb);
     }
-    seg_dt<C, EXACT>(ha, s, D, c.lam_a, ca);
-    seg_dt<C, EXACT>(hb, s, D, c.lam_b, cb);
-    const int n = s.on ? s.n : 0;
+    seg_dt<C>(A, 0, ha, s, near, c.lam_a, ca);
+    seg_dt<C>(A, 0, hb, s, near, c.lam_b, cb);
 #pragma unroll
     for (int i = 0; i < E; ++i) {
-        const bool st = EXACT && i < E - 1 ? s.on : i < n;
-        sts_if(st, c.xa + o + 4 * i, ha[i]);
-        sts_if(st, c.xb + o + 4 * i, hb[i]);
+        if (C::full || (C::fixed && i < E - 1) || i < s.n) {
+            sts(c.xa + o + 4 * i, ha[i]);
+            sts(c.xb + o + 4 * i, hb[i]);
+        }
     }
 }
 
-// One line segment of a later phase: min search along the axis (neighbour
-// stride st4 bytes) of the values at src (label 0), results to dst; cl: the
-// clip value, or with PA what is added to the line's minimum.
-template <class C, bool EXACT, bool PA>
-__device__ __forceinline__ void phase_r(const Seg &s, const Dt &D, const unsigned src, const unsigned dst,
-                                        const unsigned st4, const int lam, const int cl) {
+// Where a band's last row leaves m_b as records (p null: it does not).
+struct Rec {
+    int2 *p;  // the column's slot (label 0)
+    int tag;
+};
+
+// One line segment of a later phase (axis r): min search along the axis of the
+// values at src (label 0), results to dst; cl: the clip value, or with PA what
+// is added to the line's minimum.
+template <class C, bool PA>
+__device__ __forceinline__ void phase_r(const TeamArgs &A, const int r, const Seg &s, const bool near,
+                                        const unsigned src, const unsigned dst, const int lam, const int cl,
+                                        const Rec &rec) {
     constexpr int E = C::E;
     int h[E];
     int m = kBig;
-    unsigned a = src + 4u * (unsigned)s.off;
-    const int last = s.n - 1;
+    const unsigned st4 = 4u * (unsigned)C::stride(A, r);
+    const unsigned a = src + 4u * (unsigned)s.off, o = dst + 4u * (unsigned)s.off;
 #pragma unroll
     for (int i = 0; i < E; ++i) {
-        h[i] = lds(a);
-        if ((!EXACT || i == E - 1) && i > last) h[i] = kBig;
+        const bool maybe = C::full ? false : C::fixed ? i == E - 1 : true;
+        // past its last label a lane rereads its first
+        h[i] = lds(a + (maybe && i >= s.n ? 0u : i * st4));
+        if (maybe && i >= s.n) h[i] = kBig;
         m = min(m, h[i]);
-        // past its last label a lane rereads it
-        if (EXACT ? i < E - 2 : i < last) a += st4;
-        if (EXACT && i == E - 2 && last == E - 1) a += st4;
     }
-    seg_dt<C, EXACT>(h, s, D, lam, PA ? line_min<C>(m) + cl : cl);
-    a = dst + 4u * (unsigned)s.off;
-    const int n = s.on ? s.n : 0;
+    seg_dt<C>(A, r, h, s, near, lam, PA ? line_min<C>(m, s) + cl : cl);
 #pragma unroll
-    for (int i = 0; i < E; ++i, a += st4) sts_if(EXACT && i < E - 1 ? s.on : i < n, a, h[i]);
+    for (int i = 0; i < E; ++i)
+        if (C::full || (C::fixed && i < E - 1) || i < s.n) sts(o + i * st4, h[i]);
+    if (__builtin_expect(rec.p != nullptr, 0)) {
+        int2 *const q = rec.p + s.off;
+#pragma unroll
+        for (int i = 0; i < E; ++i)
+            if (C::full || (C::fixed && i < E - 1) || i < s.n) st_rec(q + i * C::stride(A, r), h[i], rec.tag);
+    }
+}
+
+// The same for both vectors at once (two independent chains per lane).
+template <class C, bool PA>
+__device__ __forceinline__ void phase_r2(const TeamArgs &A, const int r, const Seg &s, const bool near, const In0 &c,
+                                         const unsigned nb, const int ca, const int cb, const Rec &rec) {
+    constexpr int E = C::E;
+    int ha[E], hb[E];
+    int ma = kBig, mb = kBig;
+    const unsigned st4 = 4u * (unsigned)C::stride(A, r), o = 4u * (unsigned)s.off;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        const bool maybe = C::full ? false : C::fixed ? i == E - 1 : true;
+        const unsigned oi = o + (maybe && i >= s.n ? 0u : i * st4);
+        ha[i] = lds(c.xa + oi);
+        hb[i] = lds(c.xb + oi);
+        if (maybe && i >= s.n) ha[i] = hb[i] = kBig;
+        ma = min(ma, ha[i]);
+        mb = min(mb, hb[i]);
+    }
+    seg_dt<C>(A, r, ha, s, near, c.lam_a, PA ? line_min<C>(ma, s) + ca : ca);
+    seg_dt<C>(A, r, hb, s, near, c.lam_b, PA ? line_min<C>(mb, s) + cb : cb);
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+        if (C::full || (C::fixed && i < E - 1) || i < s.n) {
+            sts(c.xa + o + i * st4, ha[i]);
+            sts(nb + o + i * st4, hb[i]);
+        }
+    }
+    if (__builtin_expect(rec.p != nullptr, 0)) {
+        int2 *const q = rec.p + s.off;
+#pragma unroll
+        for (int i = 0; i < E; ++i)
+            if (C::full || (C::fixed && i < E - 1) || i < s.n) st_rec(q + i * C::stride(A, r), hb[i], rec.tag);
+    }
 }
 
 static __device__ __noinline__ void timed_out(int *status, volatile int *s_abort) {
@@ -415,6 +507,8 @@ static_assert(kBars * 8 <= 112, "mbarriers of a team");
 struct Row {
     int r, y, tm, wt, lane;
     bool incx, incy, has_next, to_mbox, read_c, d_ok;
+    int2 *recs;  // the band's record ring, where its last row uses one (else null)
+    int col0;    // columns of the launch before this half (tags, ring slots)
 };
 
 // arguments of a row's column loop: shared addresses of the zero vector, the
@@ -428,25 +522,35 @@ struct Row {
 template <class B, bool FIN, bool PA, bool FUSED>
 __device__ __forceinline__ void line2_row(EDP_ROW_ARGS);
 
-// A build: the cuts of the axes (C2::S = 0: two axes), exact or not.
-template <class C0_, class C1_, class C2_, bool EXACT_, int THREADS = kMaxThreads>
+// A build: the cuts of the axes (C2::S = 0: two axes).  BOTH: a warp takes both
+// vectors of its lines in the later phases, else one of them.
+struct NoCut {
+    static constexpr int S = 0, E = 1, lpw = 32, L = 1;
+    static constexpr bool fixed = true;
+    static __device__ __forceinline__ int nlines(const TeamArgs &, int) { return 1; }
+};
+template <class C0_, class C1_, class C2_, bool BOTH_, int THREADS = kMaxThreads>
 struct Build {
     using C0 = C0_;
     using C1 = C1_;
     using C2 = C2_;
-    static constexpr bool exact = EXACT_;
     static constexpr int R = C2_::S > 0 ? 3 : 2;
+    static constexpr bool both = BOTH_;
     static constexpr int threads = THREADS;  // bound of a block (registers)
+    static constexpr int extra = 0;          // working vectors of a team beside X_a, X_b
+    // labels (0: run time)
+    static constexpr int Q = C0_::fixed ? C0_::L * C1_::L * C2_::L : 0;
     template <bool FIN, bool PA, bool FUSED>
     static __device__ __forceinline__ void row(EDP_ROW_ARGS) {
         line2_row<Build, FIN, PA, FUSED>(A, w, zs, st0, xa0, xb0, bars, nx, nx_ready, wmin, wkey, bad, s_abort);
     }
-    static constexpr int extra = 0;          // working vectors of a team beside X_a, X_b
 };
-template <>
-struct Cut<0, 0> {
-    static constexpr int S = 0, E = 1, lpw = 32;
-};
+// the cuts of a fixed two- or three-axis space
+template <int Q0, int Q1, int S0, int E0, int S1, int E1, bool BOTH, int THREADS = kMaxThreads>
+using Fixed2 = Build<Cut<S0, E0, Q0, Q1, 1>, Cut<S1, E1, Q1, Q0, Q0>, NoCut, BOTH, THREADS>;
+template <int Q0, int Q1, int Q2, int S0, int E0, int S1, int E1, int S2, int E2, bool BOTH, int THREADS = kMaxThreads>
+using Fixed3 = Build<Cut<S0, E0, Q0, Q1 * Q2, 1>, Cut<S1, E1, Q1, Q0 * Q2, Q0>, Cut<S2, E2, Q2, Q0 * Q1, Q0 * Q1>, BOTH,
+                     THREADS>;
 
 // The column loop of one compute warp.
 template <class B, bool FIN, bool PA, bool FUSED>
@@ -454,22 +558,19 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
     using C0 = typename B::C0;
     using C1 = typename B::C1;
     using C2 = typename B::C2;
-    constexpr bool X = B::exact;
     constexpr int R = B::R;
-    const int W = A.W, Q = A.Q, T = A.T, tm = w.tm, wt = w.wt, lane = w.lane, y = w.y;
-    const unsigned vbytes = 4u * (unsigned)A.Qm, stb = 4u * (unsigned)stage_ints(A.Qm);
+    using CL = std::conditional_t<R == 3, C2, C1>;
+    constexpr int NV = B::both ? 1 : 2;  // warp rounds per line group in the later phases
+    const int W = A.W, T = A.T, tm = w.tm, wt = w.wt, lane = w.lane, y = w.y;
+    const int Q = B::Q ? B::Q : A.Q, Qm = B::Q ? (B::Q + 3) / 4 * 4 : A.Qm;
+    const unsigned vbytes = 4u * (unsigned)Qm, stb = 4u * (unsigned)stage_ints(Qm);
     const unsigned omc = vbytes + 16, omd = 2 * vbytes + 16, omb = 3 * vbytes + 16;
-    const int n0 = (A.ax[0].nlines + C0::lpw - 1) / C0::lpw;  // warp rounds of the phases, per vector
-    const int n1 = (A.ax[1].nlines + C1::lpw - 1) / C1::lpw, n2 = (A.ax[2].nlines + C2::lpw - 1) / C2::lpw;
-    const Seg s0 = seg_of<C0>(A.seg[0], A.ax[0], wt * C0::lpw, lane);
-    const Seg s1 = seg_of<C1>(A.seg[1], A.ax[1], (wt >= n1 ? wt - n1 : wt) * C1::lpw, lane);
+    const int n0 = (C0::nlines(A, 0) + C0::lpw - 1) / C0::lpw;  // warp rounds of the phases, per vector
+    const int n1 = (C1::nlines(A, 1) + C1::lpw - 1) / C1::lpw, nl = R == 3 ? (CL::nlines(A, 2) + CL::lpw - 1) / CL::lpw : n1;
+    const Seg s0 = seg_of<C0>(A, 0, wt * C0::lpw, lane);
+    const Seg s1 = seg_of<C1>(A, 1, (!B::both && wt >= n1 ? wt - n1 : wt) * C1::lpw, lane);
     Seg s2 = s1;
-    if (R == 3) s2 = seg_of<C2>(A.seg[2], A.ax[2], (wt >= n2 ? wt - n2 : wt) * C2::lpw, lane);
-    const bool near = A.g <= 4;
-    const Dt d0{A.seg[0].kc, A.ax[0].E, A.seg[0].nf, near && A.seg[0].kc <= 1};
-    const Dt d1{A.seg[1].kc, A.ax[1].E, A.seg[1].nf, near && A.seg[1].kc <= 1};
-    const Dt d2{A.seg[2].kc, A.ax[2].E, A.seg[2].nf, near && A.seg[2].kc <= 1};
-    const unsigned st1 = 4u * (unsigned)A.ax[1].stride, st2 = 4u * (unsigned)A.ax[2].stride;
+    if constexpr (R == 3) s2 = seg_of<CL>(A, 2, (!B::both && wt >= nl ? wt - nl : wt) * CL::lpw, lane);
     const unsigned send = 8u * (unsigned)A.nbuf;
     const unsigned xa_sum = 2 * xa0 + vbytes, xb_sum = 2 * xb0 + vbytes;  // of the two buffers
     unsigned sta = st0, sto = 0, stn = nx;  // stage of the column, its barriers, m_b in the stage of the row below
@@ -515,15 +616,14 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
             __syncwarp();
         }
         int ja = kBig, jb = kBig, sv = 0x7fffffff, sq = 0x7fffffff;
+        auto first = [&](const Seg &s, const int t) {
+            phase0<C0, FIN, PA, FUSED>(A, c, s, A.seg[0].near != 0, FUSED ? C0::pos(A, 0, s.k) : 0,
+                                       FUSED ? min(t * C0::lpw + s.l, C0::nlines(A, 0) - 1) : 0, ja, jb, sv, sq);
+        };
         if (wt < n0) {
-            phase0<C0, X, FIN, PA, FUSED>(A, c, s0, d0, seg_pos(s0.k, d0.e, d0.nf), wt * C0::lpw + (lane & (C0::lpw - 1)), ja,
-                                          jb, sv, sq);
+            first(s0, wt);
 #pragma unroll 1
-            for (int t = wt + T; __builtin_expect(t < n0, 0); t += T) {
-                const Seg s = seg_of<C0>(A.seg[0], A.ax[0], t * C0::lpw, lane);
-                phase0<C0, X, FIN, PA, FUSED>(A, c, s, d0, seg_pos(s.k, d0.e, d0.nf),
-                                              t * C0::lpw + (lane & (C0::lpw - 1)), ja, jb, sv, sq);
-            }
+            for (int t = wt + T; __builtin_expect(t < n0, 0); t += T) first(seg_of<C0>(A, 0, t * C0::lpw, lane), t);
         }
         if (FIN) {
             const int v = __reduce_min_sync(kFull, sv);
@@ -551,16 +651,27 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
             const int qm = __reduce_min_sync(kFull, v == vm ? q : 0x7fffffff);
             if (lane == 0) A.labels[(size_t)y * W + (w.incx ? xs : W - 1 - xs)] = qm;
         }
+        // a later phase: line group t (of n per vector with one vector per round)
+        auto later = [&](auto cut, const int r, const Seg &s, const int t, const int n, const unsigned nb, const int ca,
+                         const int cb, const Rec &rec) {
+            using C = decltype(cut);
+            const bool near = A.seg[r].near != 0;
+            if constexpr (B::both) {
+                phase_r2<C, PA>(A, r, s, near, c, nb, ca, cb, rec);
+            } else {
+                const bool vb = t >= n;
+                phase_r<C, PA>(A, r, s, near, vb ? c.xb : c.xa, vb ? nb : c.xa, vb ? c.lam_b : c.lam_a, vb ? cb : ca,
+                               Rec{vb ? rec.p : nullptr, rec.tag});
+            }
+        };
         int ca = PA ? c.cap_a : kBig, cb = PA ? c.cap_b : kBig;
-        if (R == 3) {
-            auto mid = [&](const Seg &s, const bool vb) {
-                phase_r<C1, X, PA>(s, d1, vb ? c.xb : c.xa, vb ? c.xb : c.xa, st1, vb ? c.lam_b : c.lam_a, vb ? cb : ca);
-            };
-            if (wt < 2 * n1) {
-                mid(s1, wt >= n1);
+        if constexpr (R == 3) {
+            if (wt < NV * n1) {
+                const Rec none{nullptr, 0};
+                later(C1(), 1, s1, wt, n1, c.xb, ca, cb, none);
 #pragma unroll 1
-                for (int t = wt + T; __builtin_expect(t < 2 * n1, 0); t += T)
-                    mid(seg_of<C1>(A.seg[1], A.ax[1], (t >= n1 ? t - n1 : t) * C1::lpw, lane), t >= n1);
+                for (int t = wt + T; __builtin_expect(t < NV * n1, 0); t += T)
+                    later(C1(), 1, seg_of<C1>(A, 1, (!B::both && t >= n1 ? t - n1 : t) * C1::lpw, lane), t, n1, c.xb, ca, cb, none);
             }
             team_sync(tm, T);
         }
@@ -568,20 +679,18 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
             ca = __reduce_min_sync(kFull, lane < T ? wmin[lane] : kBig) + c.cap_a;
             cb = __reduce_min_sync(kFull, lane < T ? wmin[kMaxT + lane] : kBig) + c.cap_b;
         }
-        {
-            using CL = std::conditional_t<R == 3, C2, C1>;
-            const Dt &dl = R == 3 ? d2 : d1;
-            const int nl = R == 3 ? n2 : n1;
-            const unsigned nb = w.to_mbox ? stn : c.xb, stl = R == 3 ? st2 : st1;
-            auto last = [&](const Seg &s, const bool vb) {
-                phase_r<CL, X, PA>(s, dl, vb ? c.xb : c.xa, vb ? nb : c.xa, stl, vb ? c.lam_b : c.lam_a, vb ? cb : ca);
-            };
-            if (wt < 2 * nl) {
-                last(s2, wt >= nl);
+        const unsigned nb = w.to_mbox ? stn : c.xb;
+        Rec rec{nullptr, 0};
+        if (__builtin_expect(w.recs != nullptr, 0)) {
+            const int s = w.col0 + xs;
+            rec.p = w.recs + (size_t)(s % A.ring) * Qm;
+            rec.tag = A.tag0 + s;
+        }
+        if (wt < NV * nl) {
+            later(CL(), R - 1, s2, wt, nl, nb, ca, cb, rec);
 #pragma unroll 1
-                for (int t = wt + T; t < 2 * nl; t += T)
-                    last(seg_of<CL>(A.seg[R - 1], A.ax[R - 1], (t >= nl ? t - nl : t) * CL::lpw, lane), t >= nl);
-            }
+            for (int t = wt + T; __builtin_expect(t < NV * nl, 0); t += T)
+                later(CL(), R - 1, seg_of<CL>(A, R - 1, (!B::both && t >= nl ? t - nl : t) * CL::lpw, lane), t, nl, nb, ca, cb, rec);
         }
         if (__builtin_expect(stop != 0, 0)) break;
         __syncwarp();
@@ -659,7 +768,7 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
     const int *const Mc = incx ? A.M[1] : A.M[0];
     int *const Mb = incy ? A.M[2] : A.M[3];
     const int *const Md = incy ? A.M[3] : A.M[2];
-    int *const ringv = reinterpret_cast<int *>(A.ll);  // [band][ring][Qm]
+    int *const ringv = reinterpret_cast<int *>(A.ll);  // copies: [band][ring][Qm] ints; records: int2
     const int col0 = h * W;                              // column counters run on over both halves
     const unsigned vbytes = 4u * (unsigned)Qm;
     const unsigned stb = 4u * (unsigned)stage_ints(Qm);  // bytes of a stage
@@ -667,7 +776,64 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
     const long long lim = A.spin_limit;
 
     if (copy && lane == 0 && wt < 2) ctl[28 + wt] = 0;
-    if (copy && row_on && lane == 0) {
+    if (copy && row_on && wt == 1 && A.rec) {
+        // ---- above, records: the whole warp polls a column's words into the stage ----
+        if (from_ring) {
+            const int2 *const recs = A.ll + (size_t)(band - 1) * ring * Qm;
+            unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride;
+            // the test hook hold_band makes one band wait for tags never written
+            const int tag0 = A.tag0 + col0 + (band == A.hold_band ? 0x20000000 : 0);
+            int si = 0, slot = col0 % ring;
+            unsigned ph = 0;
+            bool ok = true;
+            // the first half of this row still counts the ring's columns until it
+            // is complete (its out warps say so)
+            if (h == 1) ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status);
+            for (int xs = 0; xs < W && ok; ++xs) {
+                if (xs >= nst) ok = mbar_wait(bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort);
+                ok = __all_sync(kFull, ok);
+                if (!ok) break;
+                const int2 *const src = recs + (size_t)slot * Qm;
+                const unsigned dst = saddr(tb) + (unsigned)si * stb + omb;
+                const int tag = tag0 + xs;
+                constexpr int kBatch = 8;  // 16-byte loads in flight per lane
+                for (int q0 = 2 * lane; q0 < Q && ok; q0 += 64 * kBatch) {
+                    int4 v[kBatch];
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u)
+                        if (q0 + 64 * u < Q) v[u] = ld_rec2(src + q0 + 64 * u);
+#pragma unroll
+                    for (int u = 0; u < kBatch; ++u) {
+                        const int q = q0 + 64 * u;
+                        if (q >= Q || !ok) continue;
+                        for (long long n = 0; !(v[u].y == tag && (q + 1 >= Q || v[u].w == tag)); ++n) {
+                            if (n > lim || *s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) {
+                                ok = false;
+                                break;
+                            }
+                            v[u] = ld_rec2(src + q);
+                        }
+                        sts(dst + 4u * (unsigned)q, v[u].x);
+                        if (q + 1 < Q) sts(dst + 4u * (unsigned)q + 4u, v[u].z);
+                    }
+                }
+                ok = __all_sync(kFull, ok);
+                if (!ok) break;
+                if (lane == 0) {
+                    mbar_arrive(bars + kLoadB + 8 * si);
+                    ctl[29] = xs + 1;
+                    // every lane's loads of the slot have returned
+                    st_relaxed_gpu(cons, (unsigned)(col0 + xs + 1));
+                }
+                if (++si == nst) {
+                    si = 0;
+                    ph ^= 1;
+                }
+                if (++slot == ring) slot = 0;
+            }
+            if (!ok && lane == 0) timed_out(A.status, s_abort);
+        }
+    } else if (copy && row_on && lane == 0) {
         int si = 0;       // stage of the column
         unsigned ph = 0;  // its phase
         bool ok = true;
@@ -756,9 +922,24 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
             const int y_next = incy ? y + 1 : y - 1;
             const unsigned nx_bars = to_mbox ? bars_of(tm + 1) : 0;
             unsigned oph = 0;
-            // the output buffers of column p are free
+            const bool rec = A.rec != 0;
+            int room = 0;  // columns of this band's ring known to be counted by the consumer
+            // the output buffers of column xs are free, and its ring slot
+            auto ring_free = [&](int s) {
+                if (room >= s - ring + 1) return true;
+                for (long long n = 0; n <= lim; ++n) {
+                    room = (int)ld_acq_gpu(cons);
+                    if (room >= s - ring + 1) return true;
+                    if (*s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) return false;
+                    __nanosleep(20);
+                }
+                return false;
+            };
             advance(p);
-            if (p < W) mbar_arrive(bars + kReadyB + 8 * si);
+            if (p < W) {
+                if (to_ring && rec) ok = ring_free(col0 + p);
+                if (ok) mbar_arrive(bars + kReadyB + 8 * si);
+            }
             for (int xs = p; xs < W && ok; xs += 2) {
                 const int s = col0 + xs;
                 if (!(ok = mbar_wait(bars + kOutB + 8 * p, oph, lim, s_abort))) break;
@@ -773,8 +954,8 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
                                              : saddr(XB + (size_t)p * Qm);
                 if (has_next && write_b) {
                     bulk_store(Mb + ((size_t)y_next * W + x) * Qm, src, vbytes);
-                } else if (to_ring) {
-                    if (!(ok = wait_count(cons, s - ring + 1, lim, s_abort, A.status))) break;
+                } else if (to_ring && !rec) {
+                    if (!(ok = ring_free(s))) break;
                     fence_async();
                     bulk_store(ringv + ((size_t)band * ring + s % ring) * Qm, src, vbytes);
                 }
@@ -787,9 +968,10 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
                     if (to_mbox && xs + 2 >= nst &&
                         !(ok = mbar_wait(nx_bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort)))
                         break;
+                    if (to_ring && rec && !(ok = ring_free(s + 2))) break;
                     mbar_arrive(bars + kReadyB + 8 * si);
                 }
-                if (to_ring) {
+                if (to_ring && !rec) {
                     bulk_wait_all();
                     fence_async();
                     st_rel_gpu(flag + (s & 1), (unsigned)(s + 1));
@@ -803,7 +985,8 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
         }
         if (!ok) timed_out(A.status, s_abort);
     } else if (!copy && row_on) {
-        const Row w{r, y, tm, wt, lane, incx, incy, has_next, to_mbox, read_c, d_ok};
+        const Row w{r, y, tm, wt, lane, incx, incy, has_next, to_mbox, read_c, d_ok,
+                    to_ring && A.rec ? A.ll + (size_t)band * ring * Qm : nullptr, col0};
         auto run = [&](auto fin_c, auto pa_c) {
             B::template row<decltype(fin_c)::value, decltype(pa_c)::value, FUSED>(
                 A, w, saddr(zero), saddr(tb), saddr(XA), saddr(XB), bars, to_mbox ? saddr(team_of(tm + 1)) + omb : 0u,

@@ -26,6 +26,9 @@
 namespace edp {
 namespace line2 {
 
+// first position of segment k: the first nf segments hold e labels, the rest e - 1
+__device__ __forceinline__ int box_pos(int k, int e, int nf) { return k * (e - 1) + min(k, nf); }
+
 // distance transform of one vector's line segment, E labels per lane, n valid
 // (the others kBig), all carries (S <= 3)
 template <int N, int S, int E>
@@ -45,8 +48,8 @@ __device__ __forceinline__ void box_dt(int (&h)[E], const int k, const int n, co
 #pragma unroll
         for (int d = 1; d < S; ++d) {
             const int uf = __shfl_up_sync(kFull, F, d * N), ub = __shfl_down_sync(kFull, Bv, d * N);
-            if (k >= d) cf = min(cf, uf + lam * (p - seg_pos(k - d, E, nf) - E + 1));
-            if (k + d < S) cb = min(cb, ub + lam * (seg_pos(k + d, E, nf) - p - E + 1));
+            if (k >= d) cf = min(cf, uf + lam * (p - box_pos(k - d, E, nf) - E + 1));
+            if (k + d < S) cb = min(cb, ub + lam * (box_pos(k + d, E, nf) - p - E + 1));
         }
 #pragma unroll
         for (int i = 0; i < E; ++i) {
@@ -60,25 +63,24 @@ __device__ __forceinline__ void box_dt(int (&h)[E], const int k, const int n, co
 }
 
 // One vector's line after its transform: position p + i of the source line to
-// target position p + i - d (stride st bytes from dst), with clip cl; the end
+// target position p + i - d through st(position, value), with clip cl; the end
 // lanes fill the target positions beyond the source.
-template <int N, int E>
+template <int N, int E, typename St>
 __device__ __forceinline__ void box_store(const int (&h)[E], const bool on, const int p, const int n, const int d,
-                                          const unsigned dst, const unsigned st, const int lam, const int g,
-                                          const int cl) {
+                                          const int lam, const int g, const int cl, St &&st) {
 #pragma unroll
     for (int i = 0; i < E; ++i) {
         const int t = p + i - d;
-        if (on && i < n && (unsigned)t < (unsigned)N) sts(dst + st * (unsigned)t, min(h[i], cl));
+        if (on && i < n && (unsigned)t < (unsigned)N) st(t, min(h[i], cl));
     }
     if (__builtin_expect(d > 0, 0)) {  // past the source's last label
         const int last = E > 1 && n < E ? h[E > 1 ? E - 2 : 0] : h[E - 1];
         if (on && p + n == N)
-            for (int t = max(N - d, 0); t < N; ++t) sts(dst + st * (unsigned)t, min(last + lam * min(t + d - (N - 1), g), cl));
+            for (int t = max(N - d, 0); t < N; ++t) st(t, min(last + lam * min(t + d - (N - 1), g), cl));
     }
     if (__builtin_expect(d < 0, 0)) {  // before its first
         if (on && p == 0)
-            for (int t = 0; t < min(-d, N); ++t) sts(dst + st * (unsigned)t, min(h[0] + lam * min(-t - d, g), cl));
+            for (int t = 0; t < min(-d, N); ++t) st(t, min(h[0] + lam * min(-t - d, g), cl));
     }
 }
 
@@ -95,7 +97,7 @@ __device__ __forceinline__ void win_row(EDP_ROW_ARGS) {
     // lane -> segment k of line l
     const int k = lane / N, l = lane - k * N;
     const bool on = k < S;
-    const int p = on ? seg_pos(k, E, nf) : 0, n = on ? (k < nf ? E : E - 1) : 0;
+    const int p = on ? box_pos(k, E, nf) : 0, n = on ? (k < nf ? E : E - 1) : 0;
     const int r1 = ((k + 1) % S) * N + l, r2 = ((k + 2) % S) * N + l;  // the line's other lanes
     auto line_min = [&](int m) {
         if constexpr (S > 1) {
@@ -207,8 +209,12 @@ __device__ __forceinline__ void win_row(EDP_ROW_ARGS) {
         }
         box_dt<N, S, E>(ha, k, n, p, lam);
         box_dt<N, S, E>(hb, k, n, p, lam);
-        box_store<N, E>(ha, on, p, n, da0, ta + 4u * (unsigned)(N * l), 4u, lam, g, ca);
-        box_store<N, E>(hb, on, p, n, db0, tb + 4u * (unsigned)(N * l), 4u, lam, g, cb);
+        // result to a working vector or a message: position t of this line, t times st bytes from dst
+        auto to_smem = [](unsigned dst, unsigned st) {
+            return [=](int t, int v) { sts(dst + st * (unsigned)t, v); };
+        };
+        box_store<N, E>(ha, on, p, n, da0, lam, g, ca, to_smem(ta + 4u * (unsigned)(N * l), 4u));
+        box_store<N, E>(hb, on, p, n, db0, lam, g, cb, to_smem(tb + 4u * (unsigned)(N * l), 4u));
         if (FIN) {
             const int v = __reduce_min_sync(kFull, sv);
             const int q = __reduce_min_sync(kFull, sv == v ? sq : 0x7fffffff);
@@ -233,8 +239,13 @@ __device__ __forceinline__ void win_row(EDP_ROW_ARGS) {
         }
         box_dt<N, S, E>(ha, k, n, p, lam);
         box_dt<N, S, E>(hb, k, n, p, lam);
-        box_store<N, E>(ha, on, p, n, da1, xa + 4u * (unsigned)l, 4u * N, lam, g, ga);
-        box_store<N, E>(hb, on, p, n, db1, (w.to_mbox ? stn : xb) + 4u * (unsigned)l, 4u * N, lam, g, gb);
+        box_store<N, E>(ha, on, p, n, da1, lam, g, ga, to_smem(xa + 4u * (unsigned)l, 4u * N));
+        box_store<N, E>(hb, on, p, n, db1, lam, g, gb, to_smem((w.to_mbox ? stn : xb) + 4u * (unsigned)l, 4u * N));
+        if (__builtin_expect(w.recs != nullptr, 0)) {
+            const int s = w.col0 + xs, tag = A.tag0 + s;
+            int2 *const rec = w.recs + (size_t)(s % A.ring) * A.Qm + l;
+            box_store<N, E>(hb, on, p, n, db1, lam, g, gb, [&](int t, int v) { st_rec(rec + N * t, v, tag); });
+        }
         __syncwarp();
         mbar_arrive_if(lane == 0, bars + kOutB + par);
         mbar_arrive_if(lane == 0 && w.to_mbox, nx_ready + sto);
@@ -256,7 +267,7 @@ __device__ __forceinline__ void win_row(EDP_ROW_ARGS) {
 
 template <int N, int S>
 struct WinBuild {
-    static constexpr int threads = kMaxThreads;
+    static constexpr int threads = 640;  // four rows a block
     static constexpr int extra = 2;
     template <bool FIN, bool PA, bool FUSED>
     static __device__ __forceinline__ void row(EDP_ROW_ARGS) {
