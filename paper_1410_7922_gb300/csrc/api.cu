@@ -33,6 +33,10 @@ const char *g_last_kernel = "";  // scan-pass kernel of the most recent solve
 constexpr long long kSpinDefault = 4000000;
 long long g_spin_limit = kSpinDefault;  // polls before an inter-block wait gives up
 int g_hold_band = 0;     // test hook: the band whose first row waits for records never written
+// (32 problems of 96x72 with 9 x 9 labels: 5.7 ms shared, 18.8 ms alone; 12
+// problems of 160x120 to 320x240 in one, two and three axes: 103 and 31 ms; 8 of
+// 64x48 with 21 x 13 labels: 12.2 and 5.9 ms)
+constexpr int kBatchLeanPixels = 12000, kBatchGroupPixels = 2000;
 int g_batch_alone_pixels = 172800;  // batched solve: problems of this many pixels or more get their own launches
 void *const *g_prof_events = nullptr;  // optional per-pass events (profiling hook)
 int g_prof_n = 0;
@@ -306,6 +310,8 @@ struct SolvePlan {
     bool line;        // two-axis line kernel (one label line per lane)
     bool split;       // the split line kernel (two or three axes)
     int build;        // its build
+    bool axis1;       // one label axis in its frame
+    int resident;     // axis1: blocks resident at once
     int Q0, Q1;       // its label-space shape
     int nbands;
     int threads;
@@ -467,6 +473,41 @@ bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry 
     return true;
 }
 
+// One label axis in the same frame, four rows per block (a compute and four copy
+// warps each): a row below costs 0.5 us inside a block and 1.0 us between blocks,
+// a column 0.59 us against 0.55 us with one row per block (64 labels; 450x375:
+// 1.87 ms with four, 1.97 with three, 2.20 with two, 2.66 with one).
+bool plan_axis1(const int32_t *C, int *const M[4], int W, int H, const Geometry &g, const edp_params *p,
+                int32_t *labels, unsigned char *ws, SolvePlan *P) {
+    if ((long long)p->lambda * 255 > pass_line2_max_lambda() || (reinterpret_cast<uintptr_t>(C) & 15)) return false;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    const SolveLayout &L = P->L;
+    TeamArgs &a = P->ta;
+    fill_team(a, C, M, labels, ws, L, W, H, g, p);
+    a.ax[0] = TeamAxis{g.Q, 1, g.Q, 1, 1, 0, 1};
+    a.seg[0].kc = (short)pass_axis1_carry(g.Q, p->g);
+    a.T = 1;
+    a.nbuf = 4;
+    a.rec = 1;
+    const int NT = std::max(1, std::min(g_tune_rb > 0 ? std::min(g_tune_rb, 4) : 4, H));
+    a.NT = NT;
+    a.nbands = P->nbands = (H + NT - 1) / NT;
+    P->threads = pass_line2_threads(NT, 1);
+    P->smem = pass_axis1_smem(NT, L.Qm, a.nbuf, p->l1);
+    const int occ = P->smem > (size_t)kMaxSmem ? 0 : edp_pass_axis1_occupancy(g.Q, p->l1, P->threads, P->smem);
+    a.ring = line2_ring(true, a.nbuf, W, a.nbands, occ * sms);
+    if (occ < 1 || a.ring > team_ring(2 * W, kResidentMin)) {
+        memset(&P->ta, 0, sizeof P->ta);
+        return false;
+    }
+    P->resident = occ * sms;
+    P->line = P->split = P->axis1 = true;
+    return true;
+}
+
 int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_params *p, int32_t *labels,
                unsigned char *ws, SolvePlan *P, int fixed_threads = 0) {
     memset(P, 0, sizeof *P);
@@ -474,6 +515,8 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
     const SolveLayout &L = P->L;
     int *M[4];
     for (int k = 0; k < 4; ++k) M[k] = reinterpret_cast<int *>(ws + L.msg[k]);
+    if (!fixed_threads && g.R == 1 && g.Q <= 256 && !g_force_general && plan_axis1(C, M, W, H, g, p, labels, ws, P))
+        return EDP_OK;
     P->r1 = (g.R == 1 && g.Q <= 256 && !g_force_general);
     if (P->r1) {
         const int E = (g.Q + 31) / 32;
@@ -755,7 +798,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     int rc = plan_solve(C, W, H, g, p, labels, ws, &P);
     if (rc) return rc;
     if (fi) {
-        if (!P.split) return EDP_ERR_UNSUPPORTED;
+        if (!P.split || P.axis1) return EDP_ERR_UNSUPPORTED;
         P.ta.fI0 = fi->I0;
         P.ta.fI1 = fi->I1;
         P.ta.fpitch = fi->pitch;
@@ -767,7 +810,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
         P.ta.fl2 = fi->l2;
     }
     // per-edge multipliers: not the spaces of the lane-group form
-    if (wh && !P.r1 && !(P.split ? lean_space(g) : P.line || P.ta.lean)) return EDP_ERR_UNSUPPORTED;
+    if (wh && !P.r1 && !P.axis1 && !(P.split ? lean_space(g) : P.line || P.ta.lean)) return EDP_ERR_UNSUPPORTED;
     P.o.wh = P.ta.wh = wh;
     P.o.wv = P.ta.wv = wv;
     if ((rc = cuda_status(cudaMemsetAsync(ws, 0, control_bytes(P, W, g.Q), st)))) return rc;
@@ -776,7 +819,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     bool resident;  // every row band has a block at once
     if (P.split) {
-        grid_t = std::max(1, edp_pass_line2_occupancy(P.build, P.threads, P.smem)) * sms;
+        grid_t = P.axis1 ? P.resident : std::max(1, edp_pass_line2_occupancy(P.build, P.threads, P.smem)) * sms;
         // the items of both passes of a pair fill the blocks back to back, which
         // saves one drain of the resident rows per pair
         resident = P.nbands <= 4 * grid_t;
@@ -822,7 +865,9 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
                 a.band_counter = reinterpret_cast<unsigned *>(ws + P.L.counters) + slot;
                 a.grid = std::min(grid_t, P.nbands * (pairs ? 2 : 1));
                 a.trace = trace;
-                if (launch_edp_pass_line2(a, P.build, P.threads, P.smem, st)) return EDP_ERR_CUDA;
+                if (P.axis1 ? launch_edp_pass_axis1(a, P.threads, P.smem, st)
+                            : launch_edp_pass_line2(a, P.build, P.threads, P.smem, st))
+                    return EDP_ERR_CUDA;
             } else if (P.line) {
                 TeamArgs a = P.ta;
                 const int slot = it * 4 + set_launch(a, it, k, p->iters, pairs);
@@ -1271,7 +1316,7 @@ int edp_solve_images(const uint8_t *I0, const uint8_t *I1, const uint8_t *I2, in
     bool fuse = false;
     if (g_fused_cost && params->cost_mode == 0 && space->R == 2) {
         SolvePlan P;
-        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.split;
+        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.split && !P.axis1;
     }
     const FusedImages fi = fused_images(I0, I1, pitch, space, params);
     if (!fuse && (rc = run_cost(I0, I1, I2, W, H, pitch, space, params, g.Q, C, st))) return rc;
@@ -1513,7 +1558,14 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
         for (int k = first; k < first + cnt; ++k) {
             const edp_problem &pr = probs[k];
             const Geometry &g = geo[k];
-            if (g_batch_alone_pixels > 0 && (long long)pr.W * pr.H >= g_batch_alone_pixels) {
+            // two- and three-axis problems of the linear prior run on the split line
+            // kernel alone, several times faster than on the bodies of the
+            // persistent launch; only thumbnails gain by sharing it
+            // (the lane-group body, which serves any line lengths, from much smaller
+            // sizes on)
+            const bool multi = g.R >= 2 && pr.params.l1 == 1;
+            const long long alone = std::min(g_batch_alone_pixels, !multi ? INT_MAX : lean_space(g) ? kBatchLeanPixels : kBatchGroupPixels);
+            if (alone > 0 && (long long)pr.W * pr.H >= alone) {
                 unsigned char *pws = w + off;
                 int32_t *C = reinterpret_cast<int32_t *>(pws + solve_layout(pr.W, pr.H, g.Q, g.R, iters).end);
                 int rc = run_cost(pr.I0, pr.I1, pr.I2, pr.W, pr.H, pr.pitch, &pr.space, &pr.params, g.Q, C, st);

@@ -120,6 +120,12 @@ bool pass_win_built(int n);
 size_t pass_win_smem(int NT, int Qm, int nst);
 int edp_pass_win_occupancy(int n, int threads, size_t smem);
 int launch_edp_pass_win(const TeamArgs &a, int threads, size_t smem, cudaStream_t st);
+// the same for one label axis of up to 256 labels (edp_pass_axis1.cu), one
+// compute warp per row; both priors
+int pass_axis1_carry(int Q, int g);
+size_t pass_axis1_smem(int NT, int Qm, int nst, int l1);
+int edp_pass_axis1_occupancy(int Q, int l1, int threads, size_t smem);
+int launch_edp_pass_axis1(const TeamArgs &a, int threads, size_t smem, cudaStream_t st);
 // per-band stride of the line kernels' record flags and consumed counters
 // (one-lane form: one per warp of the producing / consuming team; split form:
 // flags of the even and odd columns, [2] the row's finished copy warps)

@@ -58,7 +58,9 @@
 //   records (A.rec, up to kMaxRecQ labels): the compute warps of a band's last
 //           row store {value, tag} words themselves, and the `above` warp of
 //           the next band polls them into its stage -- a matching tag carries
-//           its value, so no fence, flag or copy completion is on the path;
+//           its value, so no fence, flag or copy completion is on the path.
+//           The next column's words are requested before this one's are taken
+//           (0.70 -> 0.55 us a column at 64 labels);
 //   copies  (longer vectors, twice whose bytes would load L2): the `out` warp
 //           copies X_b to the ring (or, in the passes that keep m_b, to the
 //           message array anyway) and publishes the column when the copy has
@@ -789,33 +791,46 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
             // the first half of this row still counts the ring's columns until it
             // is complete (its out warps say so)
             if (h == 1) ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status);
+            constexpr int kBatch = 4;  // 16-byte loads per lane: 256 labels
+            auto load = [&](int4 (&v)[kBatch], const int2 *src, int q0) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u)
+                    if (q0 + 64 * u < Q) v[u] = ld_rec2(src + q0 + 64 * u);
+            };
+            // the words of labels q0, q0 + 64, ...: polled until they carry the tag
+            auto take = [&](int4 (&v)[kBatch], const int2 *src, unsigned dst, int q0, int tag) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const int q = q0 + 64 * u;
+                    if (q >= Q || !ok) continue;
+                    for (long long n = 0; !(v[u].y == tag && (q + 1 >= Q || v[u].w == tag)); ++n) {
+                        if (n > lim || *s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) {
+                            ok = false;
+                            break;
+                        }
+                        v[u] = ld_rec2(src + q);
+                    }
+                    sts(dst + 4u * (unsigned)q, v[u].x);
+                    if (q + 1 < Q) sts(dst + 4u * (unsigned)q + 4u, v[u].z);
+                }
+            };
+            int4 cur[kBatch], nxt[kBatch];  // this column's words, and the next one's already on their way
+            if (ok) load(nxt, recs + (size_t)slot * Qm, 2 * lane);
             for (int xs = 0; xs < W && ok; ++xs) {
+                const int2 *const src = recs + (size_t)slot * Qm;
+                if (++slot == ring) slot = 0;
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) cur[u] = nxt[u];
+                if (xs + 1 < W) load(nxt, recs + (size_t)slot * Qm, 2 * lane);
                 if (xs >= nst) ok = mbar_wait(bars + kEmptyB + 8 * si, ph ^ 1, lim, s_abort);
                 ok = __all_sync(kFull, ok);
                 if (!ok) break;
-                const int2 *const src = recs + (size_t)slot * Qm;
                 const unsigned dst = saddr(tb) + (unsigned)si * stb + omb;
                 const int tag = tag0 + xs;
-                constexpr int kBatch = 8;  // 16-byte loads in flight per lane
-                for (int q0 = 2 * lane; q0 < Q && ok; q0 += 64 * kBatch) {
-                    int4 v[kBatch];
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u)
-                        if (q0 + 64 * u < Q) v[u] = ld_rec2(src + q0 + 64 * u);
-#pragma unroll
-                    for (int u = 0; u < kBatch; ++u) {
-                        const int q = q0 + 64 * u;
-                        if (q >= Q || !ok) continue;
-                        for (long long n = 0; !(v[u].y == tag && (q + 1 >= Q || v[u].w == tag)); ++n) {
-                            if (n > lim || *s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) {
-                                ok = false;
-                                break;
-                            }
-                            v[u] = ld_rec2(src + q);
-                        }
-                        sts(dst + 4u * (unsigned)q, v[u].x);
-                        if (q + 1 < Q) sts(dst + 4u * (unsigned)q + 4u, v[u].z);
-                    }
+                take(cur, src, dst, 2 * lane, tag);
+                for (int q0 = 2 * lane + 64 * kBatch; q0 < Q && ok; q0 += 64 * kBatch) {
+                    load(cur, src, q0);
+                    take(cur, src, dst, q0, tag);
                 }
                 ok = __all_sync(kFull, ok);
                 if (!ok) break;
@@ -829,7 +844,6 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
                     si = 0;
                     ph ^= 1;
                 }
-                if (++slot == ring) slot = 0;
             }
             if (!ok && lane == 0) timed_out(A.status, s_abort);
         }
