@@ -1143,6 +1143,14 @@ int edp_cost_volume(const uint8_t *I0, const uint8_t *I1, const uint8_t *I2, int
     return run_cost(I0, I1, I2, W, H, pitch, space, params, g.Q, C, (cudaStream_t)stream);
 }
 
+// The scanline DP of one label axis and linear prior takes one warp per row (450x375,
+// 64 labels: 103 us against 1300 us in the general kernel, whose blocks of several
+// rows meet in barriers every column).  Up to 256 labels: one-byte back-pointers, 8
+// labels a lane.  Pinned launch shapes are the general kernel's.
+static bool scan_axis1(const Geometry &g, const edp_params *p) {
+    return g.R == 1 && g.Q <= 256 && p->l1 == 1 && g_tune_rb == 0 && g_tune_e == 0;
+}
+
 int edp_scanline_dp(const int32_t *C, int W, int H, const edp_label_space *space, const edp_params *params,
                     int32_t *labels, int64_t *row_energy, void *ws, size_t ws_bytes, edp_stream_t stream) {
     Geometry g;
@@ -1181,6 +1189,7 @@ int edp_scanline_dp(const int32_t *C, int W, int H, const edp_label_space *space
     a.l1 = params->l1;
     a.g = params->g;
     a.RB = cfg.RB;
+    if (scan_axis1(g, params)) return launch_scanline_axis1(a, st) ? EDP_ERR_CUDA : EDP_OK;
     const int grid = (H + cfg.RB - 1) / cfg.RB;
     return launch_scanline(a, cfg.em, cfg.threads, cfg.smem, grid, st) ? EDP_ERR_CUDA : EDP_OK;
 }
@@ -1223,12 +1232,13 @@ int edp_scanline_marginals(const int32_t *C, int W, int H, const edp_label_space
     a.RB = cfg.RB;
     a.no_ptr = 1;
     const int grid = (H + cfg.RB - 1) / cfg.RB;
+    const bool axis1 = scan_axis1(g, params);
     a.sums = F;
     a.reverse = 0;
-    if (launch_scanline(a, cfg.em, cfg.threads, cfg.smem, grid, st)) return EDP_ERR_CUDA;
+    if (axis1 ? launch_scanline_axis1(a, st) : launch_scanline(a, cfg.em, cfg.threads, cfg.smem, grid, st)) return EDP_ERR_CUDA;
     a.sums = B;
     a.reverse = 1;
-    if (launch_scanline(a, cfg.em, cfg.threads, cfg.smem, grid, st)) return EDP_ERR_CUDA;
+    if (axis1 ? launch_scanline_axis1(a, st) : launch_scanline(a, cfg.em, cfg.threads, cfg.smem, grid, st)) return EDP_ERR_CUDA;
     return launch_marginal_argmin(C, F, B, (long long)W * H, g.Q, labels, marginals, st) ? EDP_ERR_CUDA : EDP_OK;
 }
 

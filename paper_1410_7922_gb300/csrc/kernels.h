@@ -207,6 +207,8 @@ struct ScanArgs {
     int reverse;            // 1: the chain runs from column W-1 to 0
     int no_ptr;             // 1: no back-pointers and no backtrack (min-marginal mode)
 };
+// one label axis of up to 256 labels, truncated linear prior (one warp per row)
+int launch_scanline_axis1(const ScanArgs &a, cudaStream_t st);
 int launch_scanline(const ScanArgs &a, int em, int threads, size_t smem, int grid, cudaStream_t st);
 // S_Omega = F + B - C per pixel, lowest-index argmin (min-marginal mode)
 int launch_marginal_argmin(const int *C, const int *F, const int *B, long long npix, int Q, int *labels, int *marg,

@@ -1,0 +1,120 @@
+"""The split line kernel's frame at the sizes where its cuts, its rings and its
+dispatch can go wrong: label lines at the edges of the segment cuts, one label
+axis at the edges of the lane cuts, label boxes of every odd side, many bands
+on a small chip's worth of blocks, per-edge weights, misaligned costs (other
+kernels), the scanline DP's lane cuts and pieces.  Integer results: equal to
+the oracle bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from test_gpu_parity import dev, host, reset_tuning, sp  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def _prior(rng, mode="joint", l1=1):
+    return {"lam": int(rng.integers(0, 9)), "g": int(rng.integers(1, 7)), "l1": l1, "mode": mode}
+
+
+@pytest.mark.parametrize("mode", ["joint", "per_axis"])
+@pytest.mark.parametrize("Q", [(2, 2), (1, 9), (9, 1), (11, 7), (20, 12), (21, 13), (27, 15), (31, 19), (33, 33),
+                               (40, 33), (64, 8), (65, 40), (72, 72), (11, 7, 5), (1, 1, 6), (9, 9, 9), (16, 16, 3)])
+def test_multi_axis_cuts(edp_lib, Q, mode):
+    rng = np.random.default_rng(sum(Q) + len(mode))
+    n = int(np.prod(Q))
+    H, W = (5, 9) if n > 1000 else (14, 11)
+    for hi, g in ((21, 3), (3, 1), (200, max(Q) + 2)):  # far truncation: every segment boundary is crossed
+        C = rng.integers(0, hi, size=(H, W, n)).astype(np.int32)
+        prior = {"lam": int(rng.integers(0, 9)), "g": g, "l1": 1, "mode": mode}
+        want = oracle.edp(C, sp(Q), prior, iters=2)
+        for rows in (0, 1, 3):
+            edp_lib.set_tuning(rows, 0, 0)
+            got = host(edp_lib.solve(dev(C), sp(Q), prior, iters=2))
+            assert np.array_equal(got, want), (prior, rows, edp_lib.last_pass_kernel())
+
+
+@pytest.mark.parametrize("H,W", [(1, 1), (1, 30), (30, 1), (2, 3), (61, 5), (5, 61)])
+@pytest.mark.parametrize("Q", [(21, 13), (5, 5, 5), (37,)])
+def test_frames(edp_lib, Q, H, W):
+    """Degenerate frames, and tall ones on one row per block (many hand-offs)."""
+    rng = np.random.default_rng(H * 64 + W)
+    C = rng.integers(0, 21, size=(H, W, int(np.prod(Q)))).astype(np.int32)
+    prior = _prior(rng)
+    want = oracle.edp(C, sp(Q), prior, iters=2)
+    for rows, pairs in ((0, edp_lib.PAIRS_AUTO), (1, True), (1, False), (4, True)):
+        edp_lib.set_tuning(rows, 0, 0)
+        edp_lib.set_pass_pairs(pairs)
+        assert np.array_equal(host(edp_lib.solve(dev(C), sp(Q), prior, iters=2)), want), (rows, pairs)
+
+
+@pytest.mark.parametrize("l1", [1, 2])
+@pytest.mark.parametrize("Q", [1, 2, 15, 16, 31, 32, 33, 63, 64, 65, 127, 128, 129, 254, 255, 256])
+def test_one_axis_cuts(edp_lib, Q, l1):
+    rng = np.random.default_rng(Q * 2 + l1)
+    H, W = 11, 17
+    C = rng.integers(0, 40, size=(H, W, Q)).astype(np.int32)
+    wh, wv = (rng.integers(0, 4, size=(H, W)).astype(np.uint8) for _ in range(2))
+    for g in (1, 4, 40):
+        prior = {"lam": 3, "g": g, "l1": l1, "mode": "joint"}
+        if l1 == 2 and g == 40:
+            continue
+        want = oracle.edp(C, sp((Q,)), prior, iters=2)
+        wantw = oracle.edp_weighted(C, sp((Q,)), prior, wh, wv, iters=2)
+        for rows in (0, 1, 3):
+            edp_lib.set_tuning(rows, 0, 0)
+            assert np.array_equal(host(edp_lib.solve(dev(C), sp((Q,)), prior, iters=2)), want), (g, rows)
+        edp_lib.set_tuning(0, 0, 0)
+        assert np.array_equal(host(edp_lib.solve_weighted(dev(C), sp((Q,)), prior, dev(wh), dev(wv), 3, iters=2)), wantw)
+
+
+@pytest.mark.parametrize("Q", [(37,), (9, 9), (21, 13)])
+def test_misaligned_costs(edp_lib, Q):
+    """A cost volume 4 bytes off a 16-byte boundary gives the same labels."""
+    rng = np.random.default_rng(sum(Q))
+    n = int(np.prod(Q))
+    C = rng.integers(0, 21, size=(9, 12, n)).astype(np.int32)
+    prior = _prior(rng)
+    buf = torch.zeros(C.size + 1, dtype=torch.int32, device="cuda")
+    view = buf[1:].view(C.shape)
+    view.copy_(dev(C))
+    assert np.array_equal(host(edp_lib.solve(view, sp(Q), prior)), oracle.edp(C, sp(Q), prior))
+
+
+@pytest.mark.parametrize("mode", ["joint", "per_axis"])
+@pytest.mark.parametrize("win", [3, 5, 7, 9, 11, 13, 15])
+def test_windowed_boxes(edp_lib, win, mode):
+    """Boxes that overlap, lie far apart and are clamped at the space's ends."""
+    rng = np.random.default_rng(win)
+    Q, H, W = (33, 40), 13, 10
+    prior = {"lam": 4, "g": 3, "l1": 1, "mode": mode}
+    for spread in (2, 60):
+        centre = (rng.integers(-spread, spread + 1, size=(H, W, 2)) + 16).astype(np.int32)
+        Cw = rng.integers(0, 31, size=(H, W, win * win)).astype(np.int32)
+        want = oracle.edp_windowed(Cw, centre, sp(Q), prior, win, iters=2)
+        for rows in (0, 1, 3):
+            edp_lib.set_tuning(rows, 0, 0)
+            got = host(edp_lib.solve_windowed(dev(Cw), dev(centre), win, sp(Q), prior, iters=2))
+            assert np.array_equal(got, want), (spread, rows)
+
+
+@pytest.mark.parametrize("Q", [1, 2, 5, 63, 64, 65, 127, 128, 129, 255, 256])
+@pytest.mark.parametrize("W", [1, 2, 15, 16, 17, 66, 300])
+def test_scanline_one_axis(edp_lib, Q, W):
+    """Lane cuts (64, 128, 256 labels), the cost ring's depth, pieces of
+    back-pointers that start anywhere, heavy ties."""
+    rng = np.random.default_rng(Q * 512 + W)
+    for hi, lam, g in ((3, 1, 2), (60, 3, 5), (9, 0, 3), (250, 1, 300)):
+        C = rng.integers(0, hi, size=(5, W, Q)).astype(np.int32)
+        prior = {"lam": lam, "g": g, "l1": 1, "mode": "joint"}
+        lab, row_e = oracle.scanline_dp(C, sp((Q,)), prior, tier=1)
+        glab, grow = edp_lib.scanline_dp(dev(C), sp((Q,)), prior)
+        assert np.array_equal(host(glab), lab) and np.array_equal(host(grow), row_e), prior
+        mlab, marg = edp_lib.scanline_marginals(dev(C), sp((Q,)), prior, marginals=True)
+        edp_lib.set_tuning(2, 0, 0)  # the general kernel
+        olab, omarg = edp_lib.scanline_marginals(dev(C), sp((Q,)), prior, marginals=True)
+        glab, grow = edp_lib.scanline_dp(dev(C), sp((Q,)), prior)
+        edp_lib.set_tuning(0, 0, 0)
+        assert torch.equal(mlab, olab) and torch.equal(marg, omarg)
+        assert np.array_equal(host(glab), lab) and np.array_equal(host(grow), row_e), prior
