@@ -266,9 +266,15 @@ size_t net_status_offset();
 // tensor-core 3x3 convolution of 32 -> 32 channels (net_tc.cu): B image of a
 // layer's weights (flip: the input-gradient form), and the convolution
 // (mode 0: bias + ReLU; mode 2: input gradient masked by act > 0)
-int net_prep_tc_launch(const float *w, int flip, void *out, cudaStream_t st);
+// (of `layers` consecutive layers, 18432 bytes each)
+int net_prep_tc_launch(const float *w, int flip, int layers, void *out, cudaStream_t st);
 int net_conv_tc_launch(const void *in, int N, int H, int W, const void *wB, const float *bias, int mode, void *out,
                        const void *act, int *status, cudaStream_t st);
+// the first (5 -> 32) and last (32 -> 2) layers on the CUDA cores
+int net_edge_first(const void *in, int N, int H, int W, const float *w, const float *bias, void *out, cudaStream_t st);
+int net_edge_last(const void *in, int N, int H, int W, const float *w, const float *bias, float *out, cudaStream_t st);
+int net_edge_last_dgrad(const void *g, int N, int H, int W, const float *w, void *out, const void *act, cudaStream_t st);
+int net_edge_wgrad(const void *g, const void *x, int N, int H, int W, bool first, float *dW, float *db, cudaStream_t st);
 // weight and bias gradients of a 32 -> 32 layer on the tensor cores: each
 // block writes its partial sums to part (net_wgrad_tc_max_blocks() x
 // net_wgrad_tc_part_floats() floats), then a reduction adds them to

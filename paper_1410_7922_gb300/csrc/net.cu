@@ -41,15 +41,14 @@ __global__ void net_prep_weights(const float *w, int Co, int Ci, int flip, float
 }
 
 // 3x3 convolution, zero padding, one output pixel per thread, all output
-// channels in registers.  in: bf16 [N][H][W][Cin].  wf: float [9][Cin][Cout].
-// mode 0: out_bf = bf16(relu(z + b)); mode 1: out_f = z + b (float32);
+// channels in registers (32 -> 32, with the tensor cores off).  in: bf16
+// [N][H][W][32].  wf: float [9][32][32].  mode 0: out_bf = bf16(relu(z + b));
 // mode 2 (input gradient): out_bf = bf16(z * (act > 0)) with act bf16
-// [N][H][W][Cout] the activation at this gradient's position.
-template <int COUT>
-__global__ void __launch_bounds__(256) net_conv3x3(const __nv_bfloat16 *in, int N, int H, int W, int Cin,
+// [N][H][W][32] the activation at this gradient's position.
+__global__ void __launch_bounds__(256) net_conv3x3(const __nv_bfloat16 *in, int N, int H, int W,
                                                   const float *wf, const float *bias, int mode,
-                                                  __nv_bfloat16 *out_bf, float *out_f,
-                                                  const __nv_bfloat16 *act) {
+                                                  __nv_bfloat16 *out_bf, const __nv_bfloat16 *act) {
+    constexpr int Cin = 32, COUT = 32;
     extern __shared__ float sm[];
     // the tile's pixels are CP = Cin | 1 floats apart (odd), so that the
     // lanes of a warp, which read neighbouring pixels, hit distinct banks
@@ -90,9 +89,6 @@ __global__ void __launch_bounds__(256) net_conv3x3(const __nv_bfloat16 *in, int 
     if (mode == 0) {
 #pragma unroll
         for (int c = 0; c < COUT; ++c) out_bf[o + c] = f2bf(fmaxf(acc[c] + bias[c], 0.f));
-    } else if (mode == 1) {
-#pragma unroll
-        for (int c = 0; c < COUT; ++c) out_f[o + c] = acc[c] + bias[c];
     } else {
 #pragma unroll
         for (int c = 0; c < COUT; ++c) out_bf[o + c] = f2bf(bf2f(act[o + c]) > 0.f ? acc[c] : 0.f);
@@ -421,22 +417,13 @@ NetLayout net_layout(long long npix) {
     return L;
 }
 
-int conv(const __nv_bfloat16 *in, int N, int H, int W, int Cin, int Cout, const float *wf, const float *bias, int mode,
-         __nv_bfloat16 *out_bf, float *out_f, const __nv_bfloat16 *act, cudaStream_t st) {
+// a 32 -> 32 layer on the CUDA cores
+int conv(const __nv_bfloat16 *in, int N, int H, int W, const float *wf, const float *bias, int mode, __nv_bfloat16 *out,
+         const __nv_bfloat16 *act, cudaStream_t st) {
     dim3 grid((W + kT - 1) / kT, (H + kT - 1) / kT, N);
-    const size_t smem = (size_t)(9 * Cin * Cout + (kT + 2) * (kT + 2) * (Cin | 1)) * 4;
-    if (Cout == 32) {
-        cudaFuncSetAttribute(net_conv3x3<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        net_conv3x3<32><<<grid, kT * kT, smem, st>>>(in, N, H, W, Cin, wf, bias, mode, out_bf, out_f, act);
-    } else if (Cout == 2) {
-        cudaFuncSetAttribute(net_conv3x3<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        net_conv3x3<2><<<grid, kT * kT, smem, st>>>(in, N, H, W, Cin, wf, bias, mode, out_bf, out_f, act);
-    } else if (Cout == 5) {
-        cudaFuncSetAttribute(net_conv3x3<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        net_conv3x3<5><<<grid, kT * kT, smem, st>>>(in, N, H, W, Cin, wf, bias, mode, out_bf, out_f, act);
-    } else {
-        return -1;
-    }
+    const size_t smem = (size_t)(9 * 32 * 32 + (kT + 2) * (kT + 2) * 33) * 4;
+    cudaFuncSetAttribute(net_conv3x3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    net_conv3x3<<<grid, kT * kT, smem, st>>>(in, N, H, W, wf, bias, mode, out, act);
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 }  // namespace
@@ -459,23 +446,27 @@ int net_forward(const float *params, const void *x, int N, int H, int W, float *
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return -2;
     if (cudaMemcpyAsync(act0, x, (size_t)npix * 5 * 2, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return -2;
     float *wprep = reinterpret_cast<float *>(ws + L.wprep);
+    // the middle layers' weight images, in one launch: the backward pass's partial
+    // sums lie there later
+    unsigned char *wtc = ws + L.wpart;
+    if (g_net_tc && net_prep_tc_launch(params + param_offset(1), 0, kLayers - 2, wtc, st)) return -2;
     for (int l = 0; l < kLayers; ++l) {
         const int Ci = kChan[l], Co = kChan[l + 1];
         const float *w = params + param_offset(l);
         const float *b = w + (long long)Co * Ci * 9;
         const auto *in = reinterpret_cast<const __nv_bfloat16 *>(ws + L.act[l]);
-        if (g_net_tc && Ci == 32 && Co == 32 && l < kLayers - 1) {
-            if (net_prep_tc_launch(w, 0, ws + L.wtc, st)) return -2;
-            if (net_conv_tc_launch(in, N, H, W, ws + L.wtc, b, 0, ws + L.act[l + 1], nullptr, status, st)) return -2;
-            continue;
-        }
-        net_prep_weights<<<36, 256, 0, st>>>(w, Co, Ci, 0, wprep);
-        if (l < kLayers - 1) {
-            auto *o = reinterpret_cast<__nv_bfloat16 *>(ws + L.act[l + 1]);
-            if (conv(in, N, H, W, Ci, Co, wprep, b, 0, o, nullptr, nullptr, st)) return -2;
+        int rc = 0;
+        if (l == 0) {
+            rc = net_edge_first(in, N, H, W, w, b, ws + L.act[1], st);
+        } else if (l == kLayers - 1) {
+            rc = net_edge_last(in, N, H, W, w, b, out, st);
+        } else if (g_net_tc) {
+            rc = net_conv_tc_launch(in, N, H, W, wtc + (l - 1) * 18432, b, 0, ws + L.act[l + 1], nullptr, status, st);
         } else {
-            if (conv(in, N, H, W, Ci, Co, wprep, b, 1, nullptr, out, nullptr, st)) return -2;
+            net_prep_weights<<<36, 256, 0, st>>>(w, Co, Ci, 0, wprep);
+            rc = conv(in, N, H, W, wprep, b, 0, reinterpret_cast<__nv_bfloat16 *>(ws + L.act[l + 1]), nullptr, st);
         }
+        if (rc) return -2;
     }
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
@@ -495,7 +486,9 @@ int net_backward(const float *params, const float *out, const float *target, int
         const int Ci = kChan[l], Co = kChan[l + 1];
         const long long po = param_offset(l);
         const auto *xin = reinterpret_cast<const __nv_bfloat16 *>(ws + L.act[l]);
-        if (g_net_tc && Ci == 32 && Co == 32) {
+        if (l == 0 || l == kLayers - 1) {
+            if (net_edge_wgrad(g, xin, N, H, W, l == 0, grad + po, grad + po + (long long)Co * Ci * 9, st)) return -2;
+        } else if (g_net_tc) {
             if (net_wgrad_tc_launch(g, xin, N, H, W, reinterpret_cast<float *>(ws + L.wpart), grad + po,
                                     reinterpret_cast<int *>(ws + L.status), st))
                 return -2;
@@ -506,14 +499,16 @@ int net_backward(const float *params, const float *out, const float *target, int
         }
         if (l > 0) {
             // input gradient of layer l = output gradient of layer l-1, masked by its ReLU
-            if (g_net_tc && Ci == 32 && Co == 32) {
-                if (net_prep_tc_launch(params + po, 1, ws + L.wtc, st)) return -2;
+            if (l == kLayers - 1) {
+                if (net_edge_last_dgrad(g, N, H, W, params + po, g2, xin, st)) return -2;
+            } else if (g_net_tc) {
+                if (net_prep_tc_launch(params + po, 1, 1, ws + L.wtc, st)) return -2;
                 if (net_conv_tc_launch(g, N, H, W, ws + L.wtc, nullptr, 2, g2, xin,
                                        reinterpret_cast<int *>(ws + L.status), st))
                     return -2;
             } else {
                 net_prep_weights<<<36, 256, 0, st>>>(params + po, Co, Ci, 1, wprep);
-                if (conv(g, N, H, W, Co, Ci, wprep, nullptr, 2, g2, nullptr, xin, st)) return -2;
+                if (conv(g, N, H, W, wprep, nullptr, 2, g2, xin, st)) return -2;
             }
             auto *t = g;
             g = g2;

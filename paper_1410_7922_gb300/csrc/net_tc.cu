@@ -86,6 +86,8 @@ __device__ __forceinline__ __nv_bfloat16 f2bf(float v) { return __float2bfloat16
 // channels, K = (tap, input channel).  flip: the input-gradient form, rows
 // are the layer's input channels and K = (8 - tap, output channel).
 __global__ void net_prep_tc(const float *w, int flip, __nv_bfloat16 *out) {
+    w += (size_t)blockIdx.y * (32 * 32 * 9 + 32);  // one layer per grid row, in parameter order
+    out += (size_t)blockIdx.y * (32 * 32 * 9);
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 9 * 32 * 32; e += gridDim.x * blockDim.x) {
         const int tap = e % 9, ci = (e / 9) % 32, co = e / (9 * 32);  // w[co][ci][tap]
         const int t = flip ? 8 - tap : tap;
@@ -477,8 +479,8 @@ int net_wgrad_tc_launch(const void *g, const void *x, int N, int H, int W, float
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
-int net_prep_tc_launch(const float *w, int flip, void *out, cudaStream_t st) {
-    net_prep_tc<<<36, 256, 0, st>>>(w, flip, static_cast<__nv_bfloat16 *>(out));
+int net_prep_tc_launch(const float *w, int flip, int layers, void *out, cudaStream_t st) {
+    net_prep_tc<<<dim3(36, layers), 256, 0, st>>>(w, flip, static_cast<__nv_bfloat16 *>(out));
     return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
