@@ -9,7 +9,8 @@
 // read their weights from the parameters themselves (no preparation launch).
 //
 // With these kernels and one weight preparation for all tensor-core layers: forward,
-// 1 x 480 x 640, 264 -> 156 us; a training step, 8 x 240 x 320, 1991 -> 1048 us.
+// 1 x 480 x 640, 264 -> 156 us; a training step, 8 x 240 x 320, 1991 -> 1048 us (948
+// with one wave of blocks here and a wider sum of the partial gradients).
 // (Before: one FMA per shared-memory read, channels stored 2 bytes at a time, and a
 // block's 1440 gradient sums added to memory for every tile of 256 pixels.)
 #include <cuda_bf16.h>
@@ -298,7 +299,11 @@ int net_edge_wgrad(const void *g, const void *x, int N, int H, int W, bool first
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long n = (long long)t.x * t.y * t.z;
-    const unsigned grid = (unsigned)std::min<long long>(n, 4LL * std::max(1, sms));
+    // one wave of blocks: with a block more per SM than fit, the last ones run alone
+    const void *k = first ? (const void *)net_wgrad_edge<5, false> : (const void *)net_wgrad_edge<2, true>;
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 288, 0);
+    const unsigned grid = (unsigned)std::min<long long>(n, (long long)std::max(1, occ) * std::max(1, sms));
     const auto *gp = static_cast<const __nv_bfloat16 *>(g), *xp = static_cast<const __nv_bfloat16 *>(x);
     if (first)
         net_wgrad_edge<5, false><<<grid, 288, 0, st>>>(gp, xp, N, H, W, dW, db);
