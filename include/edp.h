@@ -133,14 +133,13 @@ size_t edp_workspace_size(int op, int W, int H, const edp_label_space *space,
  *                    scan-pass kernel instead of the warp-per-row one;
  *                    2: in addition, multi-axis spaces take its lane-group
  *                    form instead of the whole-line form;
- *                    3: two-axis spaces take the multi-axis kernel instead
- *                    of the two-axis line kernel; 4: two-axis spaces take
- *                    the line kernel wherever it is built (Q0 x Q1 = 17 x
- *                    17, 25 x 25, 33 x 33, 65 x 65 and 27 x 15, l1 = 1;
- *                    by default it serves 65 x 65); 5: as 4, with one lane
- *                    per label line also at 65 x 65 (by default the lines
- *                    of 65 x 65 are split over two lanes when lambda <=
- *                    2^30 / (34 * 255)).
+ *                    3: multi-axis spaces take the multi-axis kernel instead
+ *                    of the split line kernel (the default for l1 = 1,
+ *                    lambda <= 2^30 / (34 * 255) and a 16-byte aligned C);
+ *                    4: two-axis spaces take the line kernel with one label
+ *                    line per lane wherever it is built (Q0 x Q1 = 17 x 17,
+ *                    25 x 25, 33 x 33 and 27 x 15, l1 = 1), 65 x 65 labels
+ *                    the split one; 5: as 4, also at 65 x 65.
  * Used by the autotuner and the tests; results never depend on it.  A shape
  * the kernels cannot run makes the next solve return EDP_ERR_UNSUPPORTED.
  * Not thread-safe with concurrent solves. */
@@ -486,7 +485,10 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
  * launches in the problem's best shape (cost volume, scan passes, energy),
  * the smaller problems of a wave share one persistent launch.  0 puts every
  * problem into the persistent launch.  The default is 172,800 pixels
- * (480 x 360).  Results never depend on it.  Not thread-safe with
+ * (480 x 360).  Problems of two or three label axes with l1 = 1 run by
+ * themselves from 12,000 pixels on (2,000 where the lines are not all of 9,
+ * 17, 33 or all of 65 labels), unless min_pixels is smaller still or 0.
+ * Results never depend on it.  Not thread-safe with
  * concurrent solves. */
 int edp_set_batch_split(long long min_pixels);
 

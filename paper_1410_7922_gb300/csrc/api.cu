@@ -24,10 +24,10 @@ int g_tune_e = 0;        // labels per lane target override, scanline DP (0 = au
 int g_tune_t = 0;        // warps per row override, multi-axis scan pass (0 = automatic)
 int g_force_general = 0; // 1: one-axis problems also take the multi-axis pass kernel
 int g_generic_team = 0;  // 1: multi-axis problems take the generic team body (tests)
-int g_line_mode = 0;     // two-axis line kernel: 0 where it is faster (65-label lines), 1 off, 2 wherever built
-int g_line_split = 1;    // 65 x 65 labels: lines split over lane pairs (0: one lane per line)
+int g_line_mode = 0;     // 0 the split line kernel wherever it fits, 1 neither line kernel, 2 the one-lane line kernel wherever built
+int g_line_split = 1;    // 0: 65 x 65 labels take the one-lane line kernel, too
 int g_fused_cost = 0;    // edp_solve_images: the split line kernel computes the pair cost from the images
-int g_pass_pairs = 2;    // P1 + P2 and P3 + P4 as paired sweeps: 0 never, 1 always, 2 when every band is resident
+int g_pass_pairs = 2;    // P1 + P2 and P3 + P4 as paired sweeps: 0 never, 1 always, 2 where it is faster
 int g_last_launches = 0; // scan-pass launches of the most recent solve
 const char *g_last_kernel = "";  // scan-pass kernel of the most recent solve
 constexpr long long kSpinDefault = 4000000;

@@ -200,10 +200,10 @@ def set_tuning(rows_per_block: int = 0, labels_per_lane: int = 0, general_kernel
                warps_per_row: int = 0) -> None:
     """Launch shape of the DP kernels (0 = automatic); results never depend on it.
     general_kernel: 1 = one-axis spaces take the multi-axis kernel, 2 = and
-    multi-axis spaces its lane-group form, 3 = two-axis spaces take the
-    multi-axis kernel instead of the two-axis line kernel, 4 = two-axis spaces
-    take the line kernel wherever it is built, 5 = as 4 with one lane per label
-    line also where lines are split over lane pairs by default (65 x 65)."""
+    multi-axis spaces its lane-group form, 3 = multi-axis spaces take the
+    multi-axis kernel instead of the split line kernel, 4 = two-axis spaces
+    take the line kernel with one label line per lane wherever it is built
+    (65 x 65 labels the split one), 5 = as 4, also at 65 x 65."""
     _check(load().edp_set_tuning(int(rows_per_block), int(labels_per_lane), int(warps_per_row),
                                  int(general_kernel)), "set_tuning")
 
@@ -235,7 +235,9 @@ def set_spin_limit(polls: int = 0) -> None:
 
 def set_batch_split(min_pixels: int) -> None:
     """edp_solve_batched: problems of at least min_pixels pixels get their
-    own launches (0: every problem in the persistent launch)."""
+    own launches (0: every problem in the persistent launch).  Problems of two
+    or three label axes with l1 = 1 do from 12000 pixels on at the latest, from
+    2000 where the lines are not all of 9, 17, 33 or all of 65 labels."""
     _check(load().edp_set_batch_split(int(min_pixels)), "set_batch_split")
 
 
