@@ -118,3 +118,68 @@ def test_scanline_one_axis(edp_lib, Q, W):
         edp_lib.set_tuning(0, 0, 0)
         assert torch.equal(mlab, olab) and torch.equal(marg, omarg)
         assert np.array_equal(host(glab), lab) and np.array_equal(host(grow), row_e), prior
+
+
+@pytest.mark.parametrize("split", [0, 1500, 172800])
+def test_batch_sizes_around_the_split(edp_lib, split):
+    """Two-axis problems just below and at the sizes from which they run by
+    themselves, beside one-axis ones, under three settings of the split."""
+    rng = np.random.default_rng(3)
+    items = []
+    for W, H, Q in ((49, 40, (5, 4)), (50, 40, (5, 4)), (119, 100, (9, 9)), (120, 100, (9, 9)), (60, 50, (16,))):
+        w = dict(name=f"{W}x{H} {Q}", I2=None, space=sp(Q, [-(q // 2) for q in Q], [1] * len(Q)),
+                 prior={"lam": 5, "g": 3, "l1": 1, "mode": "per_axis"}, l2=1, cmax=20, cost_mode="pair")
+        w["I0"], w["I1"] = (rng.integers(0, 256, size=(H, W)).astype(np.uint8) for _ in range(2))
+        items.append(dict(w, I0=dev(w["I0"]), I1=dev(w["I1"]), iters=1, _w=w,
+                          labels=torch.empty((H, W), dtype=torch.int32, device="cuda"),
+                          energy4=torch.empty(4, dtype=torch.int64, device="cuda")))
+    probs = edp_lib.make_problems(items)
+    ws = torch.empty(edp_lib.batch_workspace_size(probs), dtype=torch.uint8, device="cuda")
+    edp_lib.set_batch_split(split)
+    try:
+        edp_lib.solve_batched(probs, ws)
+    finally:
+        edp_lib.set_batch_split(172800)
+    torch.cuda.synchronize()
+    for it in items:
+        w = it["_w"]
+        C = oracle.cost_volume(w["I0"], w["I1"], None, w["space"], 1, 20)
+        lab = oracle.edp(C, w["space"], w["prior"])
+        assert np.array_equal(host(it["labels"]), lab), it["name"]
+        assert tuple(int(v) for v in host(it["energy4"])) == oracle.energy(C, lab, w["space"], w["prior"]), it["name"]
+
+
+@pytest.mark.parametrize("Q,step", [((33, 5), (1, 1)), ((40,), (-1, 1)), ((65, 9), (-1, 1)), ((32, 33), (1, -1))])
+@pytest.mark.parametrize("l2", [1, 2])
+def test_pair_cost_inside_and_border(edp_lib, Q, step, l2):
+    """Frames with pixels whose whole label window lies inside the image."""
+    rng = np.random.default_rng(sum(Q) + l2)
+    space = sp(Q, [-(q // 2) * s for q, s in zip(Q, step)], step[:len(Q)])
+    I0, I1 = (rng.integers(0, 256, size=(43, 90)).astype(np.uint8) for _ in range(2))
+    got = edp_lib.cost_volume(dev(I0), dev(I1), None, space, l2, 300)
+    assert np.array_equal(host(got), oracle.cost_volume(I0, I1, None, space, l2, 300))
+
+
+def test_net_gradient_of_many_tiles_per_block(edp_lib):
+    """The gradients of four images are the mean of the single ones' (the
+    output gradients scale by a power of two, exact in bfloat16), so only the
+    order of float32 sums differs: 1e-3 of each tensor's largest entry."""
+    rng = np.random.default_rng(8)
+    N, H, W = 4, 240, 321
+    P = torch.from_numpy(rng.normal(0, 0.08, size=edp_lib.net_param_count()).astype(np.float32)).cuda()
+    x = torch.from_numpy(rng.uniform(-1, 1, size=(N, H, W, 5)).astype(np.float32)).bfloat16().cuda()
+    t = torch.from_numpy(rng.normal(0, 3, size=(N, H, W, 2)).astype(np.float32)).cuda()
+
+    def grad(a, b):
+        ws = edp_lib.net_workspace(b - a, H, W)
+        xs, ts = x[a:b].contiguous(), t[a:b].contiguous()
+        g, _ = edp_lib.net_backward(P, edp_lib.net_forward(P, xs, ws), ts, ws)
+        return g.double().cpu().numpy()
+
+    got, want = grad(0, N), sum(grad(i, i + 1) for i in range(N)) / N
+    chan = [5, 32, 32, 32, 32, 32, 2]
+    o = 0
+    for ci, co in zip(chan[:-1], chan[1:]):
+        for n in (co * ci * 9, co):
+            assert np.abs(got[o:o + n] - want[o:o + n]).max() <= 1e-3 * np.abs(want[o:o + n]).max(), (ci, co, n)
+            o += n
