@@ -789,8 +789,10 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
             unsigned ph = 0;
             bool ok = true;
             // the first half of this row still counts the ring's columns until it
-            // is complete (its out warps say so)
-            if (h == 1) ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status);
+            // is complete (its out warps say so); the lanes agree on the outcome,
+            // since they vote in every column
+            if (h == 1)
+                ok = __all_sync(kFull, wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status));
             constexpr int kBatch = 4;  // 16-byte loads per lane: 256 labels
             auto load = [&](int4 (&v)[kBatch], const int2 *src, int q0) {
 #pragma unroll
