@@ -790,13 +790,16 @@ FusedImages fused_images(const uint8_t *I0, const uint8_t *I1, int pitch, const 
 
 // wh / wv: optional per-edge prior multipliers (one-axis kernel only);
 // fi: the split line kernel computes the pair cost from these images (C is
-// not read); the caller checks that the plan is that kernel
+// not read); the caller checks that the plan is that kernel;
+// status: the word an expired wait sets, cleared by the caller (null: the
+// workspace's own, cleared here)
 int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_params *p, int32_t *labels,
               unsigned char *ws, cudaStream_t st, const uint8_t *wh = nullptr, const uint8_t *wv = nullptr,
-              const FusedImages *fi = nullptr) {
+              const FusedImages *fi = nullptr, int *status = nullptr) {
     SolvePlan P;
     int rc = plan_solve(C, W, H, g, p, labels, ws, &P);
     if (rc) return rc;
+    if (status) P.o.status = P.ta.status = status;
     if (fi) {
         if (!P.split || P.axis1) return EDP_ERR_UNSUPPORTED;
         P.ta.fI0 = fi->I0;
@@ -1391,8 +1394,9 @@ int run_wave(const edp_problem *probs_all, const Geometry *geo_all, const int *i
     int *status = reinterpret_cast<int *>(ws);
     ZeroBatch zb;
     memset(&zb, 0, sizeof zb);
-    zb.ptr[zb.n] = ws;
-    zb.bytes[zb.n++] = ctrl;
+    // (the status word in the header belongs to the whole call)
+    zb.ptr[zb.n] = ws + kHeader;
+    zb.bytes[zb.n++] = ctrl - kHeader;
     CostBatch cb;
     memset(&cb, 0, sizeof cb);
     EnergyBatch eb;
@@ -1558,6 +1562,8 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
             ++cnt;
         }
         if (cnt == 0) return EDP_ERR_WORKSPACE;
+        // one status word for every problem of the call, alone or in a shared launch
+        if (first == 0 && cudaMemsetAsync(w, 0, kHeader, st) != cudaSuccess) return EDP_ERR_CUDA;
         // regions of the chunk's problems; problems that fill the GPU on their
         // own run with their own launch shapes (one after another), the others
         // share one persistent launch
@@ -1579,7 +1585,9 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
                 unsigned char *pws = w + off;
                 int32_t *C = reinterpret_cast<int32_t *>(pws + solve_layout(pr.W, pr.H, g.Q, g.R, iters).end);
                 int rc = run_cost(pr.I0, pr.I1, pr.I2, pr.W, pr.H, pr.pitch, &pr.space, &pr.params, g.Q, C, st);
-                if (!rc) rc = run_solve(C, pr.W, pr.H, g, &pr.params, pr.labels, pws, st);
+                if (!rc)
+                    rc = run_solve(C, pr.W, pr.H, g, &pr.params, pr.labels, pws, st, nullptr, nullptr, nullptr,
+                                   reinterpret_cast<int *>(w));
                 if (!rc && pr.energy4) rc = run_energy(C, pr.labels, pr.W, pr.H, &pr.space, &pr.params, g.Q, pr.energy4, st);
                 if (rc) return rc;
             } else {

@@ -87,3 +87,44 @@ def test_batched_autotune_candidates_agree(edp_lib):
     for res in results[1:]:
         assert all(torch.equal(a, b) for a, b in zip(results[0], res))
     _check(items)
+
+
+def _random_items(edp_lib, shapes):
+    """Problems of random images: (W, H, label axes) each."""
+    rng = np.random.default_rng(len(shapes))
+    items = []
+    for W, H, Q in shapes:
+        space = {"R": len(Q), "Q": tuple(Q), "vmin": tuple(-(q // 2) for q in Q), "step": (1,) * len(Q)}
+        w = dict(name=f"{W}x{H} {Q}", I2=None, space=space, l2=1, cmax=20, cost_mode="pair",
+                 prior={"lam": 5, "g": 3, "l1": 1, "mode": "per_axis"})
+        w["I0"], w["I1"] = (rng.integers(0, 256, size=(H, W)).astype(np.uint8) for _ in range(2))
+        items.append(dict(w, I0=torch.from_numpy(w["I0"]).cuda(), I1=torch.from_numpy(w["I1"]).cuda(), iters=1, _w=w,
+                          labels=torch.zeros((H, W), dtype=torch.int32, device="cuda"),
+                          energy4=torch.empty(4, dtype=torch.int64, device="cuda")))
+    return items
+
+
+@pytest.mark.parametrize("shapes,whole", [
+    ([(50, 40, (21, 13)), (50, 40, (5, 4))], True),        # every problem on its own launches
+    ([(50, 40, (21, 13)), (40, 30, (16,))], True),         # a shared launch after one of them
+    ([(50, 40, (21, 13)), (40, 30, (16,))], False),        # the same in two waves
+])
+def test_batched_status_word(edp_lib, shapes, whole):
+    """The status word of a batch covers the problems that run on their own
+    launches: 0 after a good call on a workspace full of ones, EDP_ERR_TIMEOUT
+    after one whose first row band waited in vain, whatever ran after it."""
+    items = _random_items(edp_lib, shapes)
+    probs = edp_lib.make_problems(items)
+    n = edp_lib.batch_workspace_size(probs if whole else edp_lib.make_problems(items[:1]))
+    ws = torch.full((n,), 0xFF, dtype=torch.uint8, device="cuda")
+    for hold in (0, 1, 0):
+        try:
+            edp_lib.set_spin_limit(20000 if hold else 0)
+            edp_lib.test_hold_band(hold)
+            edp_lib.solve_batched(probs, ws)
+            assert edp_lib.get_device_status(ws) == (edp_lib.ERR_TIMEOUT if hold else 0)
+        finally:
+            edp_lib.test_hold_band(0)
+            edp_lib.set_spin_limit(0)
+        if not hold:
+            _check(items)
