@@ -313,6 +313,8 @@ struct SolvePlan {
     bool axis1;       // one label axis in its frame
     int resident;     // axis1: blocks resident at once
     int Q0, Q1;       // its label-space shape
+    // the plan's kernel can compute the pair cost from the images
+    bool fusible() const { return split && !axis1 && pass_line2_build(build).kernel(true); }
     int nbands;
     int threads;
     int em;
@@ -801,7 +803,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     if (rc) return rc;
     if (status) P.o.status = P.ta.status = status;
     if (fi) {
-        if (!P.split || P.axis1) return EDP_ERR_UNSUPPORTED;
+        if (!P.fusible()) return EDP_ERR_UNSUPPORTED;
         P.ta.fI0 = fi->I0;
         P.ta.fI1 = fi->I1;
         P.ta.fpitch = fi->pitch;
@@ -1324,12 +1326,13 @@ int edp_solve_images(const uint8_t *I0, const uint8_t *I1, const uint8_t *I2, in
     unsigned char *w = static_cast<unsigned char *>(ws);
     const ImagesLayout L = images_layout(W, H, g.Q, g.R, params->iters);
     int32_t *C = reinterpret_cast<int32_t *>(w + L.C);
-    // the pair cost of a two-axis space on the split line kernel: computed
-    // from the images inside the scan passes and the energy, no cost volume
+    // the pair cost where the split line kernel has a build for it (65 x 65
+    // labels): computed from the images inside the scan passes and the energy,
+    // no cost volume
     bool fuse = false;
     if (g_fused_cost && params->cost_mode == 0 && space->R == 2) {
         SolvePlan P;
-        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.split && !P.axis1;
+        fuse = plan_solve(C, W, H, g, params, labels, w, &P) == EDP_OK && P.fusible();
     }
     const FusedImages fi = fused_images(I0, I1, pitch, space, params);
     if (!fuse && (rc = run_cost(I0, I1, I2, W, H, pitch, space, params, g.Q, C, st))) return rc;

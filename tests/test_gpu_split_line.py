@@ -183,3 +183,40 @@ def test_net_gradient_of_many_tiles_per_block(edp_lib):
         for n in (co * ci * 9, co):
             assert np.abs(got[o:o + n] - want[o:o + n]).max() <= 1e-3 * np.abs(want[o:o + n]).max(), (ci, co, n)
             o += n
+
+
+@pytest.mark.parametrize("Q", [(33, 33), (21, 13), (9, 9), (65, 65), (40, 1), (20, 3)])
+def test_fused_cost_switch_of_every_space(edp_lib, Q):
+    """Images to labels and energy with the fused pair cost asked for: spaces
+    whose kernel has no such build get their cost volume as ever."""
+    rng = np.random.default_rng(sum(Q))
+    H, W = 14, 20
+    I0, I1 = (rng.integers(0, 256, size=(H, W)).astype(np.uint8) for _ in range(2))
+    space, prior = sp(Q, [-(q // 2) for q in Q], [1, 1]), {"lam": 4, "g": 3, "l1": 1, "mode": "per_axis"}
+    C = oracle.cost_volume(I0, I1, None, space, 1, 20)
+    want = oracle.edp(C, space, prior)
+    for shape in ((0, 0), (1, 12)):  # the planner's, and one that may need another build
+        try:
+            edp_lib.set_fused_cost(True)
+            edp_lib.set_tuning(shape[0], 0, 0, warps_per_row=shape[1])
+            lab, e = edp_lib.solve_images(dev(I0), dev(I1), None, space, prior, 1, 20)
+        finally:
+            edp_lib.set_fused_cost(False)
+            edp_lib.set_tuning(0, 0, 0)
+        assert np.array_equal(host(lab), want), shape
+        assert tuple(int(v) for v in host(e)) == oracle.energy(C, want, space, prior), shape
+
+
+def test_fused_cost_switch_and_coarse_labels(edp_lib):
+    """The coarse level of a 65 x 65 space has 33 x 33 labels."""
+    rng = np.random.default_rng(4)
+    I0, I1 = (dev(rng.integers(0, 256, size=(46, 60)).astype(np.uint8)) for _ in range(2))
+    space = sp((65, 65), (-32, -32), (1, 1))
+    prior = {"lam": 4, "g": 3, "l1": 1, "mode": "per_axis"}
+    want = edp_lib.coarse_labels(I0, I1, space, prior, 1, 20)
+    try:
+        edp_lib.set_fused_cost(True)
+        got = edp_lib.coarse_labels(I0, I1, space, prior, 1, 20)
+    finally:
+        edp_lib.set_fused_cost(False)
+    assert torch.equal(got, want)
