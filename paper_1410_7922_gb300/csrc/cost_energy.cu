@@ -227,13 +227,21 @@ __global__ void cost_pix_kernel(CostArgs A) {
     const int Q = A.Q, Q0 = A.Q0;
     const int v0 = A.vmin[0], t0 = A.step[0];
     const int v1 = A.R >= 2 ? A.vmin[1] : 0, t1 = A.R >= 2 ? A.step[1] : 0;
-    const int e0 = t0 * (Q0 - 1), e1 = A.R >= 2 ? t1 * (A.Q1 - 1) : 0;
-    const bool narrow = (long long)A.H * A.pitch <= 0x7fffffff;  // 32-bit offsets
+    // pixels whose whole window lies inside I1: [xl, xh) x [yl, yh).  In 64 bits:
+    // nothing bounds vmin
+    auto inside = [](int n, int v, int t, int L, int &lo, int &hi) {
+        const long long e = (long long)t * (L - 1), a = v + min(e, 0LL), b = v + max(e, 0LL);
+        lo = (int)min((long long)n, max(0LL, -a));
+        hi = (int)max(0LL, min((long long)n, n - b));
+    };
+    int xl, xh, yl, yh;
+    inside(A.W, v0, t0, Q0, xl, xh);
+    inside(A.H, v1, t1, A.R >= 2 ? A.Q1 : 1, yl, yh);
+    if ((long long)A.H * A.pitch > 0x7fffffff) xh = 0;  // its offsets have 32 bits
     for (long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pix < npix; pix += nw) {
         const int y = (int)(pix / A.W), x = (int)(pix - (long long)y * A.W);
         const int i0 = A.I0[(size_t)y * A.pitch + x];
-        if (narrow && x + v0 + min(e0, 0) >= 0 && x + v0 + max(e0, 0) < A.W && y + v1 + min(e1, 0) >= 0 &&
-            y + v1 + max(e1, 0) < A.H) {
+        if (x >= xl && x < xh && y >= yl && y < yh) {
             // a lane past the space's last label loads nothing: q < Q guards it
             const unsigned off = (unsigned)((y + v1) * A.pitch + x + v0 + t0 * lane);
             if (A.l2 == 1)

@@ -220,3 +220,15 @@ def test_fused_cost_switch_and_coarse_labels(edp_lib):
     finally:
         edp_lib.set_fused_cost(False)
     assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("far", [2 ** 31 - 11, 2 ** 31 - 1, -2 ** 31 + 5, -2 ** 31])
+@pytest.mark.parametrize("step", [1, -1])
+def test_pair_cost_far_displacements(edp_lib, far, step):
+    """Displacements at the ends of int32, where a window's end wraps when
+    added up in 32 bits: every label lies outside the image and costs cmax."""
+    H, W = 20, 90
+    I0, I1 = (torch.zeros((H, W), dtype=torch.uint8, device="cuda") for _ in range(2))
+    for Q, vmin in (((40,), [far]), ((40, 6), [far, 0]), ((40, 6), [0, far]), ((40, 6), [far, far])):
+        space = sp(Q, vmin, [step] * len(Q))
+        assert bool((edp_lib.cost_volume(I0, I1, None, space, 1, 7) == 7).all()), (Q, vmin)
