@@ -426,10 +426,23 @@ bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, i
 // Columns of the hand-off ring of the split line kernel's frame: some slack
 // when every band is resident, otherwise the depth that lets the first resident
 // band finish its row; with copies the consumer counts a column nst columns late.
-// (The workspace has room for team_ring(2W, kResidentMin) columns of records,
-// twice as many of plain values.)
+// (The workspace has room for team_ring(2W, kResidentMin) columns of records per
+// row, twice as many of plain values.)
 int line2_ring(bool rec, int nst, int W, int nbands, int resident) {
     return (rec ? 0 : nst) + (nbands <= resident ? 8 : team_ring(W, std::max(1, resident)));
+}
+// Columns of a ring of records: a whole row where the workspace has room, else
+// as many as it holds.  A band whose ring holds its row runs to its end
+// whatever the band below does (the second pass of a pair reuses a slot after
+// the first pass of the band below, an earlier work item), so a solve advances
+// with any number of running blocks; with fewer columns, the running bands'
+// rings together must hold a row.  (With 8 columns wherever every band had a
+// block: 64x48, 16 labels, 258 us a solve, now 251; 450x375, 64 labels, 1891 and
+// 1837; 27 x 15 labels 3447 both: clearing the longer ring costs less than
+// waiting for slots.)
+int record_ring(const SolveLayout &L, int W, int nbands) {
+    const int row = std::max(8, W);
+    return nbands < 2 ? row : (int)std::min<size_t>(row, L.ll_bytes / ((size_t)(nbands - 1) * L.Qm * 8));
 }
 bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry &g, const edp_params *p,
                 int32_t *labels, unsigned char *ws, int sms, SolvePlan *P) {
@@ -466,7 +479,7 @@ bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry 
     const int occ = edp_pass_line2_occupancy(P->build, P->threads, P->smem);
     a.rec = g.Q <= pass_line2_max_rec_labels();
     const int need = line2_ring(a.rec, S.nst, W, a.nbands, occ * sms);
-    a.ring = std::min(need, (a.rec ? 1 : 2) * team_ring(2 * W, kResidentMin));
+    a.ring = a.rec ? record_ring(L, W, a.nbands) : std::min(need, 2 * team_ring(2 * W, kResidentMin));
     if (occ < 1 || a.ring < need) {  // (cannot happen with the SMs the workspace was sized for)
         memset(&P->ta, 0, sizeof P->ta);
         P->line = P->split = false;
@@ -494,14 +507,17 @@ bool plan_axis1(const int32_t *C, int *const M[4], int W, int H, const Geometry 
     a.T = 1;
     a.nbuf = 4;
     a.rec = 1;
-    const int NT = std::max(1, std::min(g_tune_rb > 0 ? std::min(g_tune_rb, 4) : 4, H));
+    // (as many more as it takes for the workspace to hold a row of records per band:
+    // four suffice for two labels and more)
+    int NT = std::max(1, std::min(g_tune_rb > 0 ? std::min(g_tune_rb, 4) : 4, H));
+    while (NT < std::min(4, H) && record_ring(L, W, (H + NT - 1) / NT) < W) ++NT;
     a.NT = NT;
     a.nbands = P->nbands = (H + NT - 1) / NT;
     P->threads = pass_line2_threads(NT, 1);
     P->smem = pass_axis1_smem(NT, L.Qm, a.nbuf, p->l1);
     const int occ = P->smem > (size_t)kMaxSmem ? 0 : edp_pass_axis1_occupancy(g.Q, p->l1, P->threads, P->smem);
-    a.ring = line2_ring(true, a.nbuf, W, a.nbands, occ * sms);
-    if (occ < 1 || a.ring > team_ring(2 * W, kResidentMin)) {
+    a.ring = record_ring(L, W, a.nbands);
+    if (occ < 1 || a.ring < std::max(8, W)) {
         memset(&P->ta, 0, sizeof P->ta);
         return false;
     }
@@ -741,7 +757,7 @@ int plan_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_para
 // consumed-column and band counters, and the used hand-off records.
 size_t control_bytes(const SolvePlan &P, int W, int Q) {
     // plain values are published by the flags; records start without a tag
-    if (P.split) return P.L.ll + (P.ta.rec ? (size_t)P.nbands * P.ta.ring * P.L.Qm * 8 : 0);
+    if (P.split) return P.L.ll + (P.ta.rec ? (size_t)(P.nbands - 1) * P.ta.ring * P.L.Qm * 8 : 0);
     return P.r1 ? P.L.ll + (size_t)P.nbands * 2 * W * Q * 8 : P.L.ll + (size_t)P.nbands * P.ta.ring * P.L.Qm * 8;
 }
 
@@ -1678,10 +1694,10 @@ int run_windowed(TeamArgs a, const SolveLayout &L, unsigned char *w, int iters, 
     const int occ = edp_pass_win_occupancy(a.win, threads, smem);
     a.nbands = (H + NT - 1) / NT;
     a.rec = 1;
-    a.ring = line2_ring(true, a.nbuf, W, a.nbands, occ * sms);
-    if (occ < 1 || a.ring > team_ring(2 * W, kResidentMin)) return EDP_ERR_UNSUPPORTED;
+    a.ring = record_ring(L, W, a.nbands);
+    if (occ < 1 || a.ring < line2_ring(true, a.nbuf, W, a.nbands, occ * sms)) return EDP_ERR_UNSUPPORTED;
     int rc;
-    if ((rc = cuda_status(cudaMemsetAsync(w, 0, L.ll + (size_t)a.nbands * a.ring * L.Qm * 8, st)))) return rc;
+    if ((rc = cuda_status(cudaMemsetAsync(w, 0, L.ll + (size_t)(a.nbands - 1) * a.ring * L.Qm * 8, st)))) return rc;
     const bool pairs = pairs_for(a.nbands <= 4 * occ * sms);
     const int per_it = pairs ? 2 : 4;
     a.grid = std::min(a.nbands * (pairs ? 2 : 1), occ * sms);

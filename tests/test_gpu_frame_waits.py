@@ -39,3 +39,74 @@ def test_records_of_a_paired_sweep_run_out(edp_lib, Q, limit):
         got = host(edp_lib.solve(gC, sp(Q), prior, ws=ws))
         assert edp_lib.get_device_status(ws) == 0
         assert np.array_equal(got, want), band
+
+
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("Q,W,rows", [((16,), 200, 0), ((64,), 90, 2), ((37,), 60, 1), ((1,), 50, 0), ((21, 13), 12, 2)])
+def test_bands_with_a_whole_row_of_records_do_not_wait_for_those_below(edp_lib, Q, W, rows, pairs):
+    """A band whose consumer never takes a column still runs to its end (in the
+    second pass of a pair: the band above that), long before the held one
+    gives up: a solve advances with any number of running blocks."""
+    rng = np.random.default_rng(W)
+    H, hold = 40, 4
+    C = rng.integers(0, 21, size=(H, W, int(np.prod(Q)))).astype(np.int32)
+    prior = {"lam": 5, "g": 3, "l1": 1, "mode": "joint"}
+    ws = edp_lib.workspace(edp_lib.OP_SOLVE, W, H, sp(Q), prior, 1)
+    edp_lib.set_tuning(rows, 0, 0)
+    edp_lib.set_pass_pairs(pairs)
+    gC = dev(C)
+    edp_lib.solve(gC, sp(Q), prior, ws=ws)  # (the kernel is loaded before the timed launch)
+    trace = torch.zeros((H, 4), dtype=torch.int64, device="cuda")  # of the first launch
+    try:
+        edp_lib.set_trace(trace)
+        edp_lib.set_spin_limit(200000)
+        edp_lib.test_hold_band(hold)
+        edp_lib.solve(gC, sp(Q), prior, ws=ws)
+        assert edp_lib.get_device_status(ws) == edp_lib.ERR_TIMEOUT
+    finally:
+        edp_lib.test_hold_band(0)
+        edp_lib.set_spin_limit(0)
+        edp_lib.set_trace(None)
+    t = host(trace)
+    start, end = t[0, 0], t[:, 1]
+    free = hold - 1 if pairs else hold  # bands that end by themselves
+    assert (t[:hold + 1, 1] > 0).all()
+    assert end[:free].max() - start < (end[hold] - start) / 2, (end[:hold + 1] - start)
+
+
+def test_solves_at_once_on_several_streams(edp_lib):
+    """One-axis, two-axis and windowed solves in flight together, the one-axis
+    ones on streams of both priorities: labels as when each runs alone."""
+    rng = np.random.default_rng(6)
+    jobs = []
+
+    def job(Q, W, H, win=0, priority=0):
+        space, prior = sp(Q), {"lam": 8, "g": 3, "l1": 1, "mode": "per_axis"}
+        C = dev(rng.integers(0, 21, size=(H, W, win * win if win else int(np.prod(Q)))).astype(np.int32))
+        st = torch.cuda.Stream(priority=priority)
+        if win:
+            centre = dev((rng.integers(0, 3, size=(H, W, 2)) + 10).astype(np.int32))
+            ws = edp_lib.workspace_windowed(W, H, space, prior, win, 1)
+            run = lambda lab, s: edp_lib.solve_windowed(C, centre, win, space, prior, ws=ws, labels=lab, stream=s)
+        else:
+            ws = edp_lib.workspace(edp_lib.OP_SOLVE, W, H, space, prior, 1)
+            run = lambda lab, s: edp_lib.solve(C, space, prior, ws=ws, labels=lab, stream=s)
+        want = torch.empty((H, W), dtype=torch.int32, device="cuda")
+        run(want, None)
+        jobs.append((run, ws, st, want, torch.empty_like(want)))
+
+    for priority in (0, -1, 0):
+        job((64,), 300, 375, priority=priority)
+    job((33, 33), 60, 240)
+    job((27, 15), 80, 265)
+    job((33, 33), 90, 480, win=9)
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for run, ws, st, want, got in jobs:
+            with torch.cuda.stream(st):
+                got.fill_(-1)
+            run(got, st)
+    torch.cuda.synchronize()
+    for run, ws, st, want, got in jobs:
+        assert edp_lib.get_device_status(ws) == 0
+        assert torch.equal(got, want)
