@@ -205,7 +205,8 @@ int edp_set_spin_limit(long long polls);
 
 /* Test hook for the timeout path (0, the default, turns it off): in the
  * solves enqueued after the call (edp_solve, edp_solve_images,
- * edp_solve_weighted), the first row of row band `band` (> 0) waits for
+ * edp_solve_weighted, edp_solve_windowed, and the problems of
+ * edp_solve_batched that run on their own launches), the first row of row band `band` (> 0) waits for
  * hand-off data that is never published (records of a tag no producer
  * writes, or a column past the last one).  Its wait runs out after the
  * spin limit, the launch sets EDP_ERR_TIMEOUT in the device status word and

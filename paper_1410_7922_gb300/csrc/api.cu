@@ -761,6 +761,12 @@ size_t control_bytes(const SolvePlan &P, int W, int Q) {
     return P.r1 ? P.L.ll + (size_t)P.nbands * 2 * W * Q * 8 : P.L.ll + (size_t)P.nbands * P.ta.ring * P.L.Qm * 8;
 }
 
+// where scan-pass launch `launch` of a solve leaves its per-band trace (null: nowhere)
+unsigned long long *trace_of(int launch, int nbands) {
+    return g_trace && (size_t)(launch + 1) * nbands * 32 <= g_trace_bytes ? g_trace + (size_t)launch * nbands * 4
+                                                                           : nullptr;
+}
+
 bool pairs_for(bool resident) { return g_pass_pairs == 1 || (g_pass_pairs == 2 && resident); }
 
 // Launch k of iteration `it`: one pass (k = 0..3), or with paired sweeps the
@@ -870,9 +876,7 @@ int run_solve(const int32_t *C, int W, int H, const Geometry &g, const edp_param
     for (int it = 0; it < p->iters; ++it) {
         for (int k = 0; k < per_it; ++k) {
             const int launch = it * per_it + k;
-            unsigned long long *trace = (g_trace && (size_t)(launch + 1) * P.nbands * 32 <= g_trace_bytes)
-                                            ? g_trace + (size_t)launch * P.nbands * 4
-                                            : nullptr;
+            unsigned long long *trace = trace_of(launch, P.nbands);
             const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
             if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)
                 return EDP_ERR_CUDA;
@@ -1712,6 +1716,8 @@ int run_windowed(TeamArgs a, const SolveLayout &L, unsigned char *w, int iters, 
             b.rflag = reinterpret_cast<unsigned *>(w + L.lflag) + (size_t)slot * H * kLineFlagStride;
             b.tag0 = 1 + slot * W;
             b.band_counter = reinterpret_cast<unsigned *>(w + L.counters) + slot;
+            b.hold_band = g_hold_band;
+            b.trace = trace_of(launch, a.nbands);
             const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
             if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)
                 return EDP_ERR_CUDA;
@@ -1802,6 +1808,8 @@ int edp_solve_windowed(const int32_t *Cw, const int32_t *centre, int win, int W,
             b.cons = reinterpret_cast<unsigned *>(w + L.cons) + (size_t)slot * H;
             b.tag0 = 1 + slot * laps;
             b.band_counter = reinterpret_cast<unsigned *>(w + L.counters) + slot;
+            b.hold_band = g_hold_band;
+            b.trace = trace_of(launch, a.nbands);
             const bool prof = g_prof_events && 2 * launch + 1 < g_prof_n;
             if (prof && cudaEventRecord((cudaEvent_t)g_prof_events[2 * launch], st) != cudaSuccess)
                 return EDP_ERR_CUDA;

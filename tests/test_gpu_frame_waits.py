@@ -110,3 +110,34 @@ def test_solves_at_once_on_several_streams(edp_lib):
     for run, ws, st, want, got in jobs:
         assert edp_lib.get_device_status(ws) == 0
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("pairs", [False, True])
+@pytest.mark.parametrize("Q,win,l1", [((13, 13), 5, 1), ((20, 20), 9, 1), ((33, 40), 15, 1), ((13, 13), 5, 2),
+                                      ((40,), 7, 1)])
+def test_windowed_waits_run_out(edp_lib, Q, win, l1, pairs):
+    """Label boxes of two axes on the frame's rows, the other windowed forms on
+    the multi-axis kernel."""
+    rng = np.random.default_rng(win + l1)
+    H, W, R = 40, 17, len(Q)
+    centre = np.stack([rng.integers(-2, q + 2, size=(H, W)) for q in Q], axis=-1).astype(np.int32)
+    Cw = rng.integers(0, 31, size=(H, W, win ** R)).astype(np.int32)
+    prior = {"lam": 4, "g": 3, "l1": l1, "mode": "per_axis"}
+    want = oracle.edp_windowed(Cw, centre, sp(Q), prior, win, iters=1)
+    ws = edp_lib.workspace_windowed(W, H, sp(Q), prior, win, 1)
+    gC, gc = dev(Cw), dev(centre)
+    edp_lib.set_pass_pairs(pairs)
+    edp_lib.set_tuning(2, 0, 0)
+    for band in (1, 6):
+        try:
+            edp_lib.set_spin_limit(20000)
+            edp_lib.test_hold_band(band)
+            edp_lib.solve_windowed(gC, gc, win, sp(Q), prior, ws=ws)
+            assert edp_lib.get_device_status(ws) == edp_lib.ERR_TIMEOUT
+        finally:
+            edp_lib.test_hold_band(0)
+            edp_lib.set_spin_limit(0)
+        got = edp_lib.solve_windowed(gC, gc, win, sp(Q), prior, ws=ws)
+        assert edp_lib.get_device_status(ws) == 0
+        assert np.array_equal(host(got), want), band
+    assert edp_lib.last_pass_kernel() == ("edp_pass_line2_kernel" if R == 2 and l1 == 1 else "edp_pass_team_kernel")
