@@ -485,11 +485,11 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
  * `min_pixels` pixels fills the GPU by itself and is solved with its own
  * launches in the problem's best shape (cost volume, scan passes, energy),
  * the smaller problems of a wave share one persistent launch.  0 puts every
- * problem into the persistent launch.  The default is 172,800 pixels
- * (480 x 360).  Problems of two or three label axes with l1 = 1 run by
- * themselves from 12,000 pixels on (2,000 where the lines are not all of 9,
- * 17, 33 or all of 65 labels), unless min_pixels is smaller still or 0.
- * Results never depend on it.  Not thread-safe with
+ * problem into the persistent launch.  172,800 pixels (480 x 360), the
+ * default, is the measured rule: problems of two or three label axes with
+ * l1 = 1 then run by themselves from 12,000 pixels on (2,000 where the lines
+ * are not all of 9, 17, 33 or all of 65 labels).  Any other value holds for
+ * every problem.  Results never depend on it.  Not thread-safe with
  * concurrent solves. */
 int edp_set_batch_split(long long min_pixels);
 

@@ -36,8 +36,10 @@ int g_hold_band = 0;     // test hook: the band whose first row waits for record
 // (32 problems of 96x72 with 9 x 9 labels: 5.7 ms shared, 18.8 ms alone; 12
 // problems of 160x120 to 320x240 in one, two and three axes: 103 and 31 ms; 8 of
 // 64x48 with 21 x 13 labels: 12.2 and 5.9 ms)
-constexpr int kBatchLeanPixels = 12000, kBatchGroupPixels = 2000;
-int g_batch_alone_pixels = 172800;  // batched solve: problems of this many pixels or more get their own launches
+constexpr int kBatchLeanPixels = 12000, kBatchGroupPixels = 2000, kBatchPixels = 172800;
+// batched solve: problems of this many pixels or more get their own launches
+// (kBatchPixels: multi-axis ones from the sizes above on)
+int g_batch_alone_pixels = kBatchPixels;
 void *const *g_prof_events = nullptr;  // optional per-pass events (profiling hook)
 int g_prof_n = 0;
 unsigned long long *g_trace = nullptr;  // optional per-band trace buffer (device)
@@ -1602,8 +1604,8 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
             // persistent launch; only thumbnails gain by sharing it
             // (the lane-group body, which serves any line lengths, from much smaller
             // sizes on)
-            const bool multi = g.R >= 2 && pr.params.l1 == 1;
-            const long long alone = std::min(g_batch_alone_pixels, !multi ? INT_MAX : lean_space(g) ? kBatchLeanPixels : kBatchGroupPixels);
+            const bool multi = g_batch_alone_pixels == kBatchPixels && g.R >= 2 && pr.params.l1 == 1;
+            const long long alone = !multi ? g_batch_alone_pixels : lean_space(g) ? kBatchLeanPixels : kBatchGroupPixels;
             if (alone > 0 && (long long)pr.W * pr.H >= alone) {
                 unsigned char *pws = w + off;
                 int32_t *C = reinterpret_cast<int32_t *>(pws + solve_layout(pr.W, pr.H, g.Q, g.R, iters).end);

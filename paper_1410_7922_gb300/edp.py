@@ -235,9 +235,10 @@ def set_spin_limit(polls: int = 0) -> None:
 
 def set_batch_split(min_pixels: int) -> None:
     """edp_solve_batched: problems of at least min_pixels pixels get their
-    own launches (0: every problem in the persistent launch).  Problems of two
-    or three label axes with l1 = 1 do from 12000 pixels on at the latest, from
-    2000 where the lines are not all of 9, 17, 33 or all of 65 labels."""
+    own launches (0: every problem in the persistent launch).  At 172800, the
+    default, problems of two or three label axes with l1 = 1 do from 12000
+    pixels on, from 2000 where the lines are not all of 9, 17, 33 or all of 65
+    labels; any other value holds for every problem."""
     _check(load().edp_set_batch_split(int(min_pixels)), "set_batch_split")
 
 

@@ -128,3 +128,23 @@ def test_batched_status_word(edp_lib, shapes, whole):
             edp_lib.set_spin_limit(0)
         if not hold:
             _check(items)
+
+
+@pytest.mark.parametrize("split,alone", [(172800, True), (172801, False), (76800, False), (12001, False), (12000, True),
+                                         (0, False)])
+def test_batch_split_holds_for_multi_axis_problems(edp_lib, split, alone):
+    """A 120x100 problem of 9 x 9 labels runs by itself at the default setting
+    and where the setting says so, else in the shared launch (which leaves the
+    name of the last solve's kernel as it was)."""
+    items = _random_items(edp_lib, [(120, 100, (9, 9))])
+    probs = edp_lib.make_problems(items)
+    ws = torch.empty(edp_lib.batch_workspace_size(probs), dtype=torch.uint8, device="cuda")
+    edp_lib.set_tuning(0, 0, 3)
+    edp_lib.solve(torch.zeros((4, 4, 81), dtype=torch.int32, device="cuda"), items[0]["space"], items[0]["prior"])
+    edp_lib.set_tuning(0, 0, 0)
+    assert edp_lib.last_pass_kernel() == "edp_pass_team_kernel"
+    edp_lib.set_batch_split(split)
+    edp_lib.solve_batched(probs, ws)
+    assert edp_lib.last_pass_kernel() == ("edp_pass_line2_kernel" if alone else "edp_pass_team_kernel")
+    assert edp_lib.get_device_status(ws) == 0
+    _check(items)
