@@ -124,11 +124,12 @@ size_t edp_workspace_size(int op, int W, int H, const edp_label_space *space,
                           const edp_params *params);
 
 /* Process-wide launch shape of the DP kernels (0 = automatic, the default):
- *   rows_per_block   rows of the image per block (scanline DP, both
- *                    scan-pass kernels);
+ *   rows_per_block   rows of the image per block (scanline DP, scan-pass
+ *                    kernels, which take fewer where so many do not fit);
  *   labels_per_lane  target labels per lane on one label line (scanline DP);
- *   warps_per_row    warps that share one image row in the multi-axis
- *                    scan-pass kernel (1..12);
+ *   warps_per_row    warps that share one image row of a multi-axis space
+ *                    (1..12; the split line kernel's compute warps, or the
+ *                    multi-axis kernel's where that cannot run as many);
  *   general_kernel   1: one-axis label spaces also take the multi-axis
  *                    scan-pass kernel instead of the warp-per-row one;
  *                    2: in addition, multi-axis spaces take its lane-group

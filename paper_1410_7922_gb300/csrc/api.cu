@@ -398,8 +398,8 @@ bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, i
                 busy[r] = (double)n / rounds;
             }
             if (warps <= 0 && T > most) break;
-            for (int NT = 1; NT <= 8; ++NT) {
-                if (rows > 0 && NT != std::min(rows, H)) continue;
+            for (int NT = 1; NT <= pass_line2_max_rows(); ++NT) {
+                if (rows > 0 && NT != rows) continue;
                 if (NT > H || pass_line2_threads(NT, T) > B.threads) break;
                 S.NT = NT;
                 S.nst = 4;
@@ -455,9 +455,12 @@ bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry 
         return false;
     const SolveLayout &L = P->L;
     Line2Shape S;
-    // the tuning hooks' shape if there is one, else the planner's own
-    if (!line2_shape(g, p, W, H, L.Qm, sms, g_tune_rb, g_tune_t, &S) && !line2_shape(g, p, W, H, L.Qm, sms, 0, 0, &S))
-        return false;
+    // pinned rows: as many of them as fit; pinned warps no build can run: the
+    // older kernels, which run or refuse them
+    int rows = std::min(g_tune_rb, std::min(H, pass_line2_max_rows()));
+    bool have = line2_shape(g, p, W, H, L.Qm, sms, rows, g_tune_t, &S);
+    while (!have && --rows > 0) have = line2_shape(g, p, W, H, L.Qm, sms, rows, g_tune_t, &S);
+    if (!have) return false;
     P->line = P->split = true;
     P->Q0 = g.Qr[0];
     P->Q1 = g.Qr[1];

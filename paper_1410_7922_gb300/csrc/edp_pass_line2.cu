@@ -29,6 +29,7 @@ int pass_line2_builds() { return (int)(sizeof kBuilds / sizeof kBuilds[0]); }
 const Line2Build &pass_line2_build(int b) { return kBuilds[b]; }
 int pass_line2_max_rec_labels() { return line2::kMaxRecQ; }
 int pass_line2_max_warps() { return line2::kMaxT; }
+int pass_line2_max_rows() { return line2::kMaxRows; }
 int pass_line2_threads(int NT, int T) { return 32 * NT * (T + line2::kCopyWarps); }
 
 size_t pass_line2_smem(int NT, int Qm, int nst) { return ((size_t)Qm + NT * line2::team_ints(Qm, nst, 0)) * 4; }

@@ -109,6 +109,7 @@ struct Line2Build {
 int pass_line2_builds();
 const Line2Build &pass_line2_build(int b);
 int pass_line2_max_warps();
+int pass_line2_max_rows();
 int pass_line2_max_rec_labels();
 int pass_line2_threads(int NT, int T);
 size_t pass_line2_smem(int NT, int Qm, int nst);

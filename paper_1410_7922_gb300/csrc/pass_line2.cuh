@@ -87,6 +87,7 @@ namespace line2 {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kCopyWarps = 4;     // stage, above, out 0, out 1
 constexpr int kMaxT = 24;         // compute warps of a team
+constexpr int kMaxRows = 8;       // teams of a block
 constexpr int kMaxThreads = 896;  // of a block: 72 registers a thread
 constexpr int kMaxStages = 4;
 constexpr int kMaxRecQ = 512;     // labels of the record form

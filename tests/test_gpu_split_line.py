@@ -232,3 +232,22 @@ def test_pair_cost_far_displacements(edp_lib, far, step):
     for Q, vmin in (((40,), [far]), ((40, 6), [far, 0]), ((40, 6), [0, far]), ((40, 6), [far, far])):
         space = sp(Q, vmin, [step] * len(Q))
         assert bool((edp_lib.cost_volume(I0, I1, None, space, 1, 7) == 7).all()), (Q, vmin)
+
+
+@pytest.mark.parametrize("Q,rows,warps,kernel", [
+    ((33, 33), 0, 12, "edp_pass_line2_kernel"), ((33, 33), 8, 12, "edp_pass_line2_kernel"),  # one row fits
+    ((33, 33), 30, 0, "edp_pass_line2_kernel"), ((65, 65), 4, 0, "edp_pass_line2_kernel"),
+    ((17, 17, 9), 0, 8, "edp_pass_line2_kernel"),
+    ((17, 17, 9), 0, 9, "edp_pass_team_kernel"),  # 384 threads hold 8 compute and 4 copy warps
+    ((17, 17, 9), 2, 12, "edp_pass_team_kernel"),
+])
+def test_pinned_launch_shapes(edp_lib, Q, rows, warps, kernel):
+    """A pinned number of warps is never dropped: a kernel that can run it
+    does; pinned rows are an upper bound."""
+    rng = np.random.default_rng(rows + warps)
+    C = rng.integers(0, 21, size=(9, 6, int(np.prod(Q)))).astype(np.int32)
+    prior = {"lam": 4, "g": 3, "l1": 1, "mode": "per_axis"}
+    edp_lib.set_tuning(rows, 0, 0, warps_per_row=warps)
+    got = host(edp_lib.solve(dev(C), sp(Q), prior))
+    assert edp_lib.last_pass_kernel() == kernel
+    assert np.array_equal(got, oracle.edp(C, sp(Q), prior))
