@@ -130,7 +130,7 @@ def test_windowed_waits_run_out(edp_lib, Q, win, l1, pairs):
     edp_lib.set_tuning(2, 0, 0)
     for band in (1, 6):
         try:
-            edp_lib.set_spin_limit(20000)
+            edp_lib.set_spin_limit(2000)
             edp_lib.test_hold_band(band)
             edp_lib.solve_windowed(gC, gc, win, sp(Q), prior, ws=ws)
             assert edp_lib.get_device_status(ws) == edp_lib.ERR_TIMEOUT
@@ -141,3 +141,45 @@ def test_windowed_waits_run_out(edp_lib, Q, win, l1, pairs):
         assert edp_lib.get_device_status(ws) == 0
         assert np.array_equal(host(got), want), band
     assert edp_lib.last_pass_kernel() == ("edp_pass_line2_kernel" if R == 2 and l1 == 1 else "edp_pass_team_kernel")
+
+
+@pytest.mark.parametrize("pairs", [0, 1])
+@pytest.mark.parametrize("Q", [(16,), (200,), (9, 9), (33, 33), (65, 65), (11, 7, 5), (9, 9, 9), (17, 17, 9)])
+def test_waits_of_the_default_kernels_run_out(edp_lib, Q, pairs):
+    """The kernels the planner picks: records up to 512 labels, copies above."""
+    rng = np.random.default_rng(sum(Q))
+    H, W = (20, 8) if np.prod(Q) > 2000 else (36, 20)
+    C = rng.integers(0, 21, size=(H, W, int(np.prod(Q)))).astype(np.int32)
+    prior = {"lam": 5, "g": 3, "l1": 1, "mode": "per_axis"}
+    gC, ws = dev(C), edp_lib.workspace(edp_lib.OP_SOLVE, W, H, sp(Q), prior, 1)
+    edp_lib.set_pass_pairs(pairs)
+    try:
+        edp_lib.set_spin_limit(20000)
+        edp_lib.test_hold_band(2)
+        edp_lib.solve(gC, sp(Q), prior, ws=ws)
+        assert edp_lib.get_device_status(ws) == edp_lib.ERR_TIMEOUT
+    finally:
+        edp_lib.test_hold_band(0)
+        edp_lib.set_spin_limit(0)
+    got = host(edp_lib.solve(gC, sp(Q), prior, ws=ws))
+    assert edp_lib.get_device_status(ws) == 0
+    assert edp_lib.last_pass_kernel() == "edp_pass_line2_kernel"
+    assert np.array_equal(got, oracle.edp(C, sp(Q), prior, tier=1))
+
+
+def test_more_bands_than_blocks(edp_lib):
+    """Tall frames of one row per block: rings shorter than a row between bands
+    that run one after another, label boxes and split lines."""
+    rng = np.random.default_rng(5)
+    H, W, Q = 6000, 12, (13, 11)
+    prior = {"lam": 4, "g": 3, "l1": 1, "mode": "per_axis"}
+    centre = np.stack([rng.integers(-2, q + 2, size=(H, W)) for q in Q], axis=-1).astype(np.int32)
+    Cw = rng.integers(0, 31, size=(H, W, 25)).astype(np.int32)
+    C = rng.integers(0, 21, size=(H, W, 143)).astype(np.int32)
+    want_w = oracle.edp_windowed(Cw, centre, sp(Q), prior, 5, iters=1)
+    want = oracle.edp(C, sp(Q), prior, tier=1)
+    edp_lib.set_tuning(1, 0, 0)
+    for pairs in (0, 1, 2):
+        edp_lib.set_pass_pairs(pairs)
+        assert np.array_equal(host(edp_lib.solve_windowed(dev(Cw), dev(centre), 5, sp(Q), prior, iters=1)), want_w), pairs
+        assert np.array_equal(host(edp_lib.solve(dev(C), sp(Q), prior)), want), pairs
