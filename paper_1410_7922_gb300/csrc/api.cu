@@ -390,11 +390,10 @@ bool line2_shape(const Geometry &g, const edp_params *p, int W, int H, int Qm, i
             double ins[3] = {0, 0, 0}, busy[3] = {0, 0, 0};  // instructions of a warp, warps at work, per phase
             int most = 1;
             for (int r = 0; r < g.R; ++r) {
-                const int lpw = S.seg[r].lpw, nv = r > 0 && !B.both ? 2 : 1;
-                const int n = nv * ((g.Q / g.Qr[r] + lpw - 1) / lpw);
+                const int lpw = S.seg[r].lpw, n = (g.Q / g.Qr[r] + lpw - 1) / lpw;
                 const int rounds = (n + T - 1) / T;
                 most = std::max(most, n);
-                ins[r] = rounds * ((r == 0 ? 22.0 : B.both ? 17.0 : 9.0) * B.E[r] * (B.Q[0] ? 1.0 : 1.4) + 45.0);
+                ins[r] = rounds * ((r == 0 ? 22.0 : 17.0) * B.E[r] * (B.Q[0] ? 1.0 : 1.4) + 45.0);
                 busy[r] = (double)n / rounds;
             }
             if (warps <= 0 && T > most) break;

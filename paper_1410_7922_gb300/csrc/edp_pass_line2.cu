@@ -8,20 +8,20 @@ namespace edp {
 
 static const Line2Build kBuilds[] = {
     // the label spaces of the repository's workloads and tests
-    {{65, 65, 1}, {5, 5, 0}, {13, 13, 0}, true, 480, line2_k0},
-    {{33, 33, 1}, {3, 3, 0}, {11, 11, 0}, true, 512, line2_k1},
-    {{27, 15, 1}, {3, 3, 0}, {9, 5, 0}, true, 512, line2_k2},
-    {{25, 25, 1}, {3, 3, 0}, {9, 9, 0}, true, 512, line2_k3},
-    {{17, 17, 1}, {1, 1, 0}, {17, 17, 0}, true, 512, line2_k4},
-    {{9, 9, 1}, {3, 3, 0}, {3, 3, 0}, true, 640, line2_k5},
-    {{17, 17, 9}, {1, 1, 1}, {17, 17, 9}, true, 384, line2_k6},
-    {{9, 9, 9}, {1, 1, 1}, {9, 9, 9}, true, 512, line2_k7},
+    {{65, 65, 1}, {5, 5, 0}, {13, 13, 0}, 480, line2_k0},
+    {{33, 33, 1}, {3, 3, 0}, {11, 11, 0}, 512, line2_k1},
+    {{27, 15, 1}, {3, 3, 0}, {9, 5, 0}, 512, line2_k2},
+    {{25, 25, 1}, {3, 3, 0}, {9, 9, 0}, 512, line2_k3},
+    {{17, 17, 1}, {1, 1, 0}, {17, 17, 0}, 512, line2_k4},
+    {{9, 9, 1}, {3, 3, 0}, {3, 3, 0}, 640, line2_k5},
+    {{17, 17, 9}, {1, 1, 1}, {17, 17, 9}, 384, line2_k6},
+    {{9, 9, 9}, {1, 1, 1}, {9, 9, 9}, 512, line2_k7},
     // any line lengths up to segments x labels
-    {{0, 0, 0}, {2, 2, 0}, {8, 8, 0}, true, 512, line2_k8},
-    {{0, 0, 0}, {4, 2, 0}, {8, 8, 0}, true, 512, line2_k9},
-    {{0, 0, 0}, {4, 4, 0}, {8, 8, 0}, true, 512, line2_k10},
-    {{0, 0, 0}, {8, 8, 0}, {9, 9, 0}, true, 512, line2_k11},
-    {{0, 0, 0}, {2, 2, 2}, {8, 8, 8}, true, 512, line2_k12},
+    {{0, 0, 0}, {2, 2, 0}, {8, 8, 0}, 512, line2_k8},
+    {{0, 0, 0}, {4, 2, 0}, {8, 8, 0}, 512, line2_k9},
+    {{0, 0, 0}, {4, 4, 0}, {8, 8, 0}, 512, line2_k10},
+    {{0, 0, 0}, {8, 8, 0}, {9, 9, 0}, 512, line2_k11},
+    {{0, 0, 0}, {2, 2, 2}, {8, 8, 8}, 512, line2_k12},
 };
 
 int pass_line2_max_lambda() { return line2::kMaxLambda; }

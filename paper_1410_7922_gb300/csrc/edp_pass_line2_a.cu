@@ -3,7 +3,7 @@
 
 namespace edp {
 
-void *line2_k0(bool fused) { return line2_kernel<Fixed2<65, 65, 5, 13, 5, 13, true, 480>, true>(fused); }
-void *line2_k5(bool fused) { return line2_kernel<Fixed2<9, 9, 3, 3, 3, 3, true, 640>, false>(fused); }
+void *line2_k0(bool fused) { return line2_kernel<Fixed2<65, 65, 5, 13, 5, 13, 480>, true>(fused); }
+void *line2_k5(bool fused) { return line2_kernel<Fixed2<9, 9, 3, 3, 3, 3, 640>, false>(fused); }
 
 }  // namespace edp

@@ -3,8 +3,8 @@
 
 namespace edp {
 
-void *line2_k3(bool fused) { return line2_kernel<Fixed2<25, 25, 3, 9, 3, 9, true, 512>, false>(fused); }
-void *line2_k4(bool fused) { return line2_kernel<Fixed2<17, 17, 1, 17, 1, 17, true, 512>, false>(fused); }
-void *line2_k8(bool fused) { return line2_kernel<Build<Cut<2, 8>, Cut<2, 8>, NoCut, true, 512>, false>(fused); }
+void *line2_k3(bool fused) { return line2_kernel<Fixed2<25, 25, 3, 9, 3, 9, 512>, false>(fused); }
+void *line2_k4(bool fused) { return line2_kernel<Fixed2<17, 17, 1, 17, 1, 17, 512>, false>(fused); }
+void *line2_k8(bool fused) { return line2_kernel<Build<Cut<2, 8>, Cut<2, 8>, NoCut, 512>, false>(fused); }
 
 }  // namespace edp

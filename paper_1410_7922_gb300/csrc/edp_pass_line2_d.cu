@@ -3,7 +3,7 @@
 
 namespace edp {
 
-void *line2_k6(bool fused) { return line2_kernel<Fixed3<17, 17, 9, 1, 17, 1, 17, 1, 9, true, 384>, false>(fused); }
-void *line2_k7(bool fused) { return line2_kernel<Fixed3<9, 9, 9, 1, 9, 1, 9, 1, 9, true, 512>, false>(fused); }
+void *line2_k6(bool fused) { return line2_kernel<Fixed3<17, 17, 9, 1, 17, 1, 17, 1, 9, 384>, false>(fused); }
+void *line2_k7(bool fused) { return line2_kernel<Fixed3<9, 9, 9, 1, 9, 1, 9, 1, 9, 512>, false>(fused); }
 
 }  // namespace edp

@@ -102,7 +102,6 @@ int pass_line2_max_lambda();
 struct Line2Build {
     int Q[3];                // the label space it is for (0: any whose lines fit)
     int S[3], E[3];          // segments per line and labels per lane of each axis (S = 0: no such axis)
-    bool both;               // both vectors per warp in the later phases
     int threads;             // bound of a block
     void *(*kernel)(bool fused);
 };

@@ -26,9 +26,10 @@
 //   phase 0   the halved sums of Eq. DP_2D_base on lines of axis 0, both
 //             vectors in the same lane (the five inputs are read once), the
 //             min search along axis 0, results to X_a (next buffer) and X_b;
-//   barrier;  phases 1 .. R-1: the same along axes 1, 2 in place, one vector
-//             per warp (a barrier between them); the last one leaves m_a in X_a
-//             and m_b in the stage of the row below (or in X_b, shipped by `out`);
+//   barrier;  phases 1 .. R-1: the same along axes 1, 2 in place, again both
+//             vectors in the same lane (a barrier between them); the last one
+//             leaves m_a in X_a and m_b in the stage of the row below (or in
+//             X_b, shipped by `out`);
 //   barrier.
 // The min search is separable, so the order of the axes changes no value.
 //
@@ -432,42 +433,13 @@ struct Rec {
     int tag;
 };
 
-// One line segment of a later phase (axis r): min search along the axis of the
-// values at src (label 0), results to dst; cl: the clip value, or with PA what
-// is added to the line's minimum.
+// One line segment of both vectors in a later phase (axis r; two independent
+// chains per lane): min search along the axis of the values in X_a and X_b,
+// m_a's back to X_a, m_b's to nb; ca, cb: the clip values, or with PA what is
+// added to the line's minima.
 template <class C, bool PA>
-__device__ __forceinline__ void phase_r(const TeamArgs &A, const int r, const Seg &s, const bool near,
-                                        const unsigned src, const unsigned dst, const int lam, const int cl,
-                                        const Rec &rec) {
-    constexpr int E = C::E;
-    int h[E];
-    int m = kBig;
-    const unsigned st4 = 4u * (unsigned)C::stride(A, r);
-    const unsigned a = src + 4u * (unsigned)s.off, o = dst + 4u * (unsigned)s.off;
-#pragma unroll
-    for (int i = 0; i < E; ++i) {
-        const bool maybe = C::full ? false : C::fixed ? i == E - 1 : true;
-        // past its last label a lane rereads its first
-        h[i] = lds(a + (maybe && i >= s.n ? 0u : i * st4));
-        if (maybe && i >= s.n) h[i] = kBig;
-        m = min(m, h[i]);
-    }
-    seg_dt<C>(A, r, h, s, near, lam, PA ? line_min<C>(m, s) + cl : cl);
-#pragma unroll
-    for (int i = 0; i < E; ++i)
-        if (C::full || (C::fixed && i < E - 1) || i < s.n) sts(o + i * st4, h[i]);
-    if (__builtin_expect(rec.p != nullptr, 0)) {
-        int2 *const q = rec.p + s.off;
-#pragma unroll
-        for (int i = 0; i < E; ++i)
-            if (C::full || (C::fixed && i < E - 1) || i < s.n) st_rec(q + i * C::stride(A, r), h[i], rec.tag);
-    }
-}
-
-// The same for both vectors at once (two independent chains per lane).
-template <class C, bool PA>
-__device__ __forceinline__ void phase_r2(const TeamArgs &A, const int r, const Seg &s, const bool near, const In0 &c,
-                                         const unsigned nb, const int ca, const int cb, const Rec &rec) {
+__device__ __forceinline__ void phase_r(const TeamArgs &A, const int r, const Seg &s, const bool near, const In0 &c,
+                                        const unsigned nb, const int ca, const int cb, const Rec &rec) {
     constexpr int E = C::E;
     int ha[E], hb[E];
     int ma = kBig, mb = kBig;
@@ -527,20 +499,18 @@ struct Row {
 template <class B, bool FIN, bool PA, bool FUSED>
 __device__ __forceinline__ void line2_row(EDP_ROW_ARGS);
 
-// A build: the cuts of the axes (C2::S = 0: two axes).  BOTH: a warp takes both
-// vectors of its lines in the later phases, else one of them.
+// A build: the cuts of the axes (C2::S = 0: two axes).
 struct NoCut {
     static constexpr int S = 0, E = 1, lpw = 32, L = 1;
     static constexpr bool fixed = true;
     static __device__ __forceinline__ int nlines(const TeamArgs &, int) { return 1; }
 };
-template <class C0_, class C1_, class C2_, bool BOTH_, int THREADS = kMaxThreads>
+template <class C0_, class C1_, class C2_, int THREADS = kMaxThreads>
 struct Build {
     using C0 = C0_;
     using C1 = C1_;
     using C2 = C2_;
     static constexpr int R = C2_::S > 0 ? 3 : 2;
-    static constexpr bool both = BOTH_;
     static constexpr int threads = THREADS;  // bound of a block (registers)
     static constexpr int extra = 0;          // working vectors of a team beside X_a, X_b
     // labels (0: run time)
@@ -551,10 +521,10 @@ struct Build {
     }
 };
 // the cuts of a fixed two- or three-axis space
-template <int Q0, int Q1, int S0, int E0, int S1, int E1, bool BOTH, int THREADS = kMaxThreads>
-using Fixed2 = Build<Cut<S0, E0, Q0, Q1, 1>, Cut<S1, E1, Q1, Q0, Q0>, NoCut, BOTH, THREADS>;
-template <int Q0, int Q1, int Q2, int S0, int E0, int S1, int E1, int S2, int E2, bool BOTH, int THREADS = kMaxThreads>
-using Fixed3 = Build<Cut<S0, E0, Q0, Q1 * Q2, 1>, Cut<S1, E1, Q1, Q0 * Q2, Q0>, Cut<S2, E2, Q2, Q0 * Q1, Q0 * Q1>, BOTH,
+template <int Q0, int Q1, int S0, int E0, int S1, int E1, int THREADS = kMaxThreads>
+using Fixed2 = Build<Cut<S0, E0, Q0, Q1, 1>, Cut<S1, E1, Q1, Q0, Q0>, NoCut, THREADS>;
+template <int Q0, int Q1, int Q2, int S0, int E0, int S1, int E1, int S2, int E2, int THREADS = kMaxThreads>
+using Fixed3 = Build<Cut<S0, E0, Q0, Q1 * Q2, 1>, Cut<S1, E1, Q1, Q0 * Q2, Q0>, Cut<S2, E2, Q2, Q0 * Q1, Q0 * Q1>,
                      THREADS>;
 
 // The column loop of one compute warp.
@@ -565,7 +535,6 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
     using C2 = typename B::C2;
     constexpr int R = B::R;
     using CL = std::conditional_t<R == 3, C2, C1>;
-    constexpr int NV = B::both ? 1 : 2;  // warp rounds per line group in the later phases
     const int W = A.W, T = A.T, tm = w.tm, wt = w.wt, lane = w.lane, y = w.y;
     const int Q = B::Q ? B::Q : A.Q, Qm = B::Q ? (B::Q + 3) / 4 * 4 : A.Qm;
     const unsigned vbytes = 4u * (unsigned)Qm, stb = 4u * (unsigned)stage_ints(Qm);
@@ -573,9 +542,9 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
     const int n0 = (C0::nlines(A, 0) + C0::lpw - 1) / C0::lpw;  // warp rounds of the phases, per vector
     const int n1 = (C1::nlines(A, 1) + C1::lpw - 1) / C1::lpw, nl = R == 3 ? (CL::nlines(A, 2) + CL::lpw - 1) / CL::lpw : n1;
     const Seg s0 = seg_of<C0>(A, 0, wt * C0::lpw, lane);
-    const Seg s1 = seg_of<C1>(A, 1, (!B::both && wt >= n1 ? wt - n1 : wt) * C1::lpw, lane);
+    const Seg s1 = seg_of<C1>(A, 1, wt * C1::lpw, lane);
     Seg s2 = s1;
-    if constexpr (R == 3) s2 = seg_of<CL>(A, 2, (!B::both && wt >= nl ? wt - nl : wt) * CL::lpw, lane);
+    if constexpr (R == 3) s2 = seg_of<CL>(A, 2, wt * CL::lpw, lane);
     const unsigned send = 8u * (unsigned)A.nbuf;
     const unsigned xa_sum = 2 * xa0 + vbytes, xb_sum = 2 * xb0 + vbytes;  // of the two buffers
     unsigned sta = st0, sto = 0, stn = nx;  // stage of the column, its barriers, m_b in the stage of the row below
@@ -656,27 +625,18 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
             const int qm = __reduce_min_sync(kFull, v == vm ? q : 0x7fffffff);
             if (lane == 0) A.labels[(size_t)y * W + (w.incx ? xs : W - 1 - xs)] = qm;
         }
-        // a later phase: line group t (of n per vector with one vector per round)
-        auto later = [&](auto cut, const int r, const Seg &s, const int t, const int n, const unsigned nb, const int ca,
-                         const int cb, const Rec &rec) {
-            using C = decltype(cut);
-            const bool near = A.seg[r].near != 0;
-            if constexpr (B::both) {
-                phase_r2<C, PA>(A, r, s, near, c, nb, ca, cb, rec);
-            } else {
-                const bool vb = t >= n;
-                phase_r<C, PA>(A, r, s, near, vb ? c.xb : c.xa, vb ? nb : c.xa, vb ? c.lam_b : c.lam_a, vb ? cb : ca,
-                               Rec{vb ? rec.p : nullptr, rec.tag});
-            }
+        // a line group of a later phase
+        auto later = [&](auto cut, const int r, const Seg &s, const unsigned nb, const int ca, const int cb, const Rec &rec) {
+            phase_r<decltype(cut), PA>(A, r, s, A.seg[r].near != 0, c, nb, ca, cb, rec);
         };
         int ca = PA ? c.cap_a : kBig, cb = PA ? c.cap_b : kBig;
         if constexpr (R == 3) {
-            if (wt < NV * n1) {
+            if (wt < n1) {
                 const Rec none{nullptr, 0};
-                later(C1(), 1, s1, wt, n1, c.xb, ca, cb, none);
+                later(C1(), 1, s1, c.xb, ca, cb, none);
 #pragma unroll 1
-                for (int t = wt + T; __builtin_expect(t < NV * n1, 0); t += T)
-                    later(C1(), 1, seg_of<C1>(A, 1, (!B::both && t >= n1 ? t - n1 : t) * C1::lpw, lane), t, n1, c.xb, ca, cb, none);
+                for (int t = wt + T; __builtin_expect(t < n1, 0); t += T)
+                    later(C1(), 1, seg_of<C1>(A, 1, t * C1::lpw, lane), c.xb, ca, cb, none);
             }
             team_sync(tm, T);
         }
@@ -691,11 +651,11 @@ __device__ __forceinline__ void line2_row(EDP_ROW_ARGS) {
             rec.p = w.recs + (size_t)(s % A.ring) * Qm;
             rec.tag = A.tag0 + s;
         }
-        if (wt < NV * nl) {
-            later(CL(), R - 1, s2, wt, nl, nb, ca, cb, rec);
+        if (wt < nl) {
+            later(CL(), R - 1, s2, nb, ca, cb, rec);
 #pragma unroll 1
-            for (int t = wt + T; __builtin_expect(t < NV * nl, 0); t += T)
-                later(CL(), R - 1, seg_of<CL>(A, R - 1, (!B::both && t >= nl ? t - nl : t) * CL::lpw, lane), t, nl, nb, ca, cb, rec);
+            for (int t = wt + T; __builtin_expect(t < nl, 0); t += T)
+                later(CL(), R - 1, seg_of<CL>(A, R - 1, t * CL::lpw, lane), nb, ca, cb, rec);
         }
         if (__builtin_expect(stop != 0, 0)) break;
         __syncwarp();
