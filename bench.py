@@ -228,7 +228,10 @@ KERNEL_SOURCES = {
     "edp_pass_r1_kernel": ("pass_r1.cuh", "edp_pass_r1.cu", "common.cuh"),
     "edp_pass_team_kernel": ("pass_team.cuh", "edp_pass_team.cu", "common.cuh"),
     "edp_pass_line_kernel": ("pass_line.cuh", "edp_pass_line.cu", "common.cuh"),
-    "edp_pass_line2_kernel": ("pass_line2.cuh", "pass_axis1.cuh", "line2_kernel.cuh", "edp_pass_line2.cu", "common.cuh"),
+    "edp_pass_line2_kernel": ("pass_line2.cuh", "pass_axis1.cuh", "pass_win.cuh", "line2_kernel.cuh", "line2_builds.h",
+                              "edp_pass_line2.cu", "edp_pass_line2_a.cu", "edp_pass_line2_b.cu", "edp_pass_line2_c.cu",
+                              "edp_pass_line2_d.cu", "edp_pass_line2_e.cu", "edp_pass_line2_f.cu", "edp_pass_axis1.cu",
+                              "edp_pass_win.cu", "common.cuh"),
 }
 
 
