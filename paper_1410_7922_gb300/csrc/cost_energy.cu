@@ -2,6 +2,8 @@
 // (Eq. GE_objective_function) kernels, sm_103a.
 #include <cstdint>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -220,28 +222,35 @@ __device__ __forceinline__ void cost_pix_inside(const CostArgs &A, unsigned off,
     for (; q < Q; q += 32, out += 32) *out = cost(__ldg(A.I1 + next()));
 }
 
-__global__ void cost_pix_kernel(CostArgs A) {
+// The pixels whose whole window lies inside I1: [xl, xh) x [yl, yh).
+struct InsideRect {
+    int xl, xh, yl, yh;
+};
+// In 64 bits: nothing bounds vmin.
+static InsideRect inside_rect(const CostArgs &a) {
+    auto span = [](int n, int v, int t, int L, int &lo, int &hi) {
+        const long long e = (long long)t * (L - 1), first = v + std::min(e, 0LL), last = v + std::max(e, 0LL);
+        lo = (int)std::min((long long)n, std::max(0LL, -first));
+        hi = (int)std::max(0LL, std::min((long long)n, n - last));
+    };
+    InsideRect r;
+    span(a.W, a.vmin[0], a.step[0], a.Q0, r.xl, r.xh);
+    span(a.H, a.R >= 2 ? a.vmin[1] : 0, a.R >= 2 ? a.step[1] : 0, a.R >= 2 ? a.Q1 : 1, r.yl, r.yh);
+    if ((long long)a.H * a.pitch > 0x7fffffff) r.xh = 0;  // the loop's offsets have 32 bits
+    return r;
+}
+
+__global__ void cost_pix_kernel(CostArgs A, InsideRect in) {
     const int lane = threadIdx.x & 31;
     const long long npix = (long long)A.W * A.H;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     const int Q = A.Q, Q0 = A.Q0;
     const int v0 = A.vmin[0], t0 = A.step[0];
     const int v1 = A.R >= 2 ? A.vmin[1] : 0, t1 = A.R >= 2 ? A.step[1] : 0;
-    // pixels whose whole window lies inside I1: [xl, xh) x [yl, yh).  In 64 bits:
-    // nothing bounds vmin
-    auto inside = [](int n, int v, int t, int L, int &lo, int &hi) {
-        const long long e = (long long)t * (L - 1), a = v + min(e, 0LL), b = v + max(e, 0LL);
-        lo = (int)min((long long)n, max(0LL, -a));
-        hi = (int)max(0LL, min((long long)n, n - b));
-    };
-    int xl, xh, yl, yh;
-    inside(A.W, v0, t0, Q0, xl, xh);
-    inside(A.H, v1, t1, A.R >= 2 ? A.Q1 : 1, yl, yh);
-    if ((long long)A.H * A.pitch > 0x7fffffff) xh = 0;  // its offsets have 32 bits
     for (long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; pix < npix; pix += nw) {
         const int y = (int)(pix / A.W), x = (int)(pix - (long long)y * A.W);
         const int i0 = A.I0[(size_t)y * A.pitch + x];
-        if (x >= xl && x < xh && y >= yl && y < yh) {
+        if (x >= in.xl && x < in.xh && y >= in.yl && y < in.yh) {
             // a lane past the space's last label loads nothing: q < Q guards it
             const unsigned off = (unsigned)((y + v1) * A.pitch + x + v0 + t0 * lane);
             if (A.l2 == 1)
@@ -291,7 +300,7 @@ int launch_cost(const CostArgs &a, cudaStream_t st) {
         long long blocks = ((long long)a.W * a.H + 7) / 8;
         if (blocks > 152LL * 16) blocks = 152LL * 16;
         if (blocks < 1) blocks = 1;
-        cost_pix_kernel<<<(unsigned)blocks, threads, 0, st>>>(a);
+        cost_pix_kernel<<<(unsigned)blocks, threads, 0, st>>>(a, inside_rect(a));
         return cudaGetLastError() == cudaSuccess ? 0 : -2;
     }
     if ((reinterpret_cast<uintptr_t>(a.C) & 15) == 0) {  // four entries per thread and step
