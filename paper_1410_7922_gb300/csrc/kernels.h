@@ -52,7 +52,7 @@ struct TeamArgs {
     int *M[4];              // [H][W][Qm] messages into each pixel from +x, -x, +y, -y
     int *labels;            // [H][W], written by the final pass
     int2 *ll;               // [nbands][ring][Qm] {value, tag} records between bands
-    unsigned *cons;         // [nbands] columns of each band's records consumed ([nbands][8] per warp: line kernels)
+    unsigned *cons;         // [nbands] columns of each band's records consumed (line kernels: [nbands][8], per warp or per half of a pair)
     unsigned *rflag;        // line kernels: [nbands][8] columns of records each producing warp has written
     unsigned *band_counter;
     int *status;

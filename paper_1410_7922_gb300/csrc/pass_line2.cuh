@@ -67,8 +67,8 @@
 //           message array anyway) and publishes the column when the copy has
 //           completed (release at GPU scope); `above` acquires that and copies.
 // A ring slot is written again once the consumer has counted its column (cons).
-// Both halves of a pair count into one word; the second half's block starts after
-// the first half's last count (rflag).
+// The halves of a pair count in a word each, since nothing orders the stores of their
+// two blocks; the larger count holds.
 // (33 x 33 labels, 320x240: 3.7 ms a solve with copies, T = 0.9 us a column but
 // 4 us a hand-off, and at most one column a microsecond through it.)
 //
@@ -728,10 +728,6 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
     const bool has_next = r + 1 < H;
     const bool to_mbox = has_next && tm + 1 < NT, to_ring = has_next && tm + 1 == NT;
     const bool from_ring = r > 0 && tm == 0;
-    // warps that say when they are done with a row of a pair's first half: both
-    // out warps, and `above`, whose count of consumed columns the second half's
-    // (another block's) continues
-    const int row_done = 2 + (from_ring ? 1 : 0);
     const bool d_ok = A.read_d && (incy ? y + 1 < H : y - 1 >= 0);
     int *const Ma = incx ? A.M[0] : A.M[1];
     const int *const Mc = incx ? A.M[1] : A.M[0];
@@ -749,18 +745,17 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
         // ---- above, records: the whole warp polls a column's words into the stage ----
         if (from_ring) {
             const int2 *const recs = A.ll + (size_t)(band - 1) * ring * Qm;
-            unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride;
+            unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride + h;
             // the test hook hold_band makes one band wait for tags never written
             const int tag0 = A.tag0 + col0 + (band == A.hold_band ? 0x20000000 : 0);
             int si = 0, slot = col0 % ring;
             unsigned ph = 0;
             bool ok = true;
             // the first half of this row still counts the ring's columns until it
-            // is complete; the lanes agree on the outcome, since they vote in every
-            // column
+            // is complete (its out warps say so); the lanes agree on the outcome,
+            // since they vote in every column
             if (h == 1)
-                ok = __all_sync(kFull,
-                                wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, row_done, lim, s_abort, A.status));
+                ok = __all_sync(kFull, wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status));
             constexpr int kBatch = 4;  // 16-byte loads per lane: 256 labels
             auto load = [&](int4 (&v)[kBatch], const int2 *src, int q0) {
 #pragma unroll
@@ -815,12 +810,7 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
                     ph ^= 1;
                 }
             }
-            if (lane == 0) {
-                if (!ok)
-                    timed_out(A.status, s_abort);
-                else if (A.pair && h == 0)
-                    add_rel_gpu(A.rflag + (size_t)r * kLineFlagStride + 2, 1u);
-            }
+            if (!ok && lane == 0) timed_out(A.status, s_abort);
         }
     } else if (copy && row_on && lane == 0) {
         int si = 0;       // stage of the column
@@ -835,8 +825,8 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
         };
         if (wt == 0) {
             // ---- stage: C, m_c, m_d of every column ----
-            if (h == 1) {  // this row of the first half is complete
-                ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, row_done, lim, s_abort, A.status);
+            if (h == 1) {  // this row of the first half is complete (both its out warps)
+                ok = wait_count(A.rflag + (size_t)r * kLineFlagStride + 2, 2, lim, s_abort, A.status);
                 fence_async();
             }
             const size_t NQ = (size_t)W * H * Q;
@@ -869,7 +859,7 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
             // ---- above: m_b of every column the previous band published ----
             if (from_ring) {
                 const unsigned *const flag = A.rflag + (size_t)(band - 1) * kLineFlagStride;
-                unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride;
+                unsigned *const cons = A.cons + (size_t)(band - 1) * kLineFlagStride + h;
                 // the test hook hold_band makes one band wait for a column never published
                 const int hold = band == A.hold_band ? 0x20000000 : 0;
                 int seen[2] = {0, 0};  // published columns as last read, even / odd
@@ -902,7 +892,6 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
                 for (int xs = max(0, W - nst); xs < W && ok; ++xs)
                     ok = mbar_wait(bars + kEmptyB + 8 * (xs % nst), (xs / nst) & 1, lim, s_abort);
                 if (ok) st_relaxed_gpu(cons, (unsigned)(col0 + W));
-                if (ok && A.pair && h == 0) add_rel_gpu(A.rflag + (size_t)r * kLineFlagStride + 2, 1u);
             }
         } else {
             // ---- out p: the finished columns p, p + 2, ... ----
@@ -918,7 +907,8 @@ __device__ __forceinline__ bool line2_item(const TeamArgs &A, const int h, const
             auto ring_free = [&](int s) {
                 if (room >= s - ring + 1) return true;
                 for (long long n = 0; n <= lim; ++n) {
-                    room = (int)ld_acq_gpu(cons);
+                    const uint2 v = ld_acq_gpu2(cons);
+                    room = (int)max(v.x, v.y);
                     if (room >= s - ring + 1) return true;
                     if (*s_abort || ((n & 63) == 63 && *(volatile int *)A.status != 0)) return false;
                     __nanosleep(20);
