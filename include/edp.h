@@ -20,6 +20,15 @@
  *    on the host before anything is enqueued.  Errors detected on the device
  *    (a bounded inter-block wait that expired) are written to the status word
  *    inside the workspace; read it with edp_get_device_status.
+ *  - The row bands of a solve hand their results on through rings in the
+ *    workspace.  With one label axis of up to 256 labels a ring holds a
+ *    whole row, and the solve advances with any number of running blocks.
+ *    The other solves count on the blocks of a launch, at most one wave of
+ *    the device's SMs, running together once earlier work has drained: solves
+ *    on streams of equal priority take turns, but one that is kept from most
+ *    of the SMs for longer than the spin limit (by a stream of higher
+ *    priority, or by a partition of the device smaller than the number of
+ *    SMs it reports) ends with EDP_ERR_TIMEOUT in its status word.
  *
  * Label space (Sec. 2, Eq. v_r_x_d)
  * ----------------------------------
@@ -154,20 +163,23 @@ int edp_set_tuning(int rows_per_block, int labels_per_lane, int warps_per_row, i
  * iteration instead of four).
  *   mode 0: one launch per pass;
  *   mode 1: paired sweeps always;
- *   mode 2 (the default): paired sweeps when every row band of the problem
- *           has a block at once (a paired band holds its block twice as long,
- *           which costs more than it saves when bands wait for blocks);
- *           edp_solve_batched pairs only in mode 1 (its bands share the
- *           blocks).
+ *   mode 2 (the default): paired sweeps where they are faster.  The split
+ *           line kernel (general_kernel 0) pairs as long as the bands of one
+ *           pass fill the blocks at most four times over; the other kernels
+ *           when every row band has a block at once (a paired band holds its
+ *           block twice as long, which costs more than it saves when bands
+ *           wait for blocks); the persistent launch of edp_solve_batched
+ *           pairs only in mode 1 (its bands share the blocks).
  * Results never depend on it.  Returns EDP_ERR_INVALID_ARG unless mode is 0,
  * 1 or 2.  Not thread-safe with concurrent solves. */
 int edp_set_pass_pairs(int mode);
 
-/* Cost volume of edp_solve_images / edp_solve_images_host.  1: where the
- * pair cost (Eq. Cost_value, cost_mode pair) of a two-axis label space runs
- * on the split form of the two-axis line kernel, the scan passes and the
- * energy compute C(x, q) from the images as they need it and no cost volume
- * is built (the values are those edp_cost_volume stores).  0 (the default):
+/* Cost volume of edp_solve_images / edp_solve_images_host (and the coarse
+ * solve of edp_coarse_labels).  1: where the split line kernel has a build
+ * for the pair cost (Eq. Cost_value, cost_mode pair; 65 x 65 labels), the scan
+ * passes and the energy compute C(x, q) from the images as they need it and
+ * no cost volume is built (the values are those edp_cost_volume stores);
+ * every other space gets its cost volume.  0 (the default):
  * the cost volume is always built first (measured faster at 640x480 with
  * 65 x 65 labels: the scan passes' byte loads of 65 image rows per column
  * cost more than the cost volume saves).  Results never depend on it.
@@ -415,9 +427,9 @@ int edp_net_centres(const float *out, int n, const edp_label_space *space, int32
  * floor(vmax/2) per axis), and each full-resolution pixel (x, y) gets the
  * label of coarse pixel (x/2, y/2) with its offsets doubled and clamped into
  * `space`.  labels: device int32 [H][W] (linear label index of `space`).
- * ws: edp_workspace_size(EDP_OP_COARSE, ...) bytes, 256-byte aligned; the
- * coarse solve's status word is the workspace's first int at offset 256.
- * Errors as edp_solve_images. */
+ * ws: edp_workspace_size(EDP_OP_COARSE, ...) bytes, 256-byte aligned (the
+ * status word of the coarse solve lies inside its part of it, not at the
+ * start).  Errors as edp_solve_images. */
 int edp_coarse_labels(const uint8_t *I0, const uint8_t *I1, int W, int H, int pitch, const edp_label_space *space,
                       const edp_params *params, int32_t *labels, void *ws, size_t ws_bytes, edp_stream_t stream);
 
@@ -469,17 +481,17 @@ typedef struct {
 size_t edp_batch_workspace_size(const edp_problem *probs, int n);
 
 /* Batched form of edp_solve_images for many independent problems of uneven
- * sizes and label spaces (one, two and three label axes mixed).  Per wave of
- * resident problems: one launch zeroes the control words, one builds every
- * cost volume, ONE persistent launch runs every scan pass of every problem
- * (work items (pass, problem, row band) taken in order from a global queue,
- * with bounded waits on the previous band and the previous pass of the same
- * problem), and one launch evaluates every energy.  Results are identical to
- * solving each problem alone.  `probs` is host memory and is read during the
+ * sizes and label spaces (one, two and three label axes mixed).  Problems at
+ * or above the sizes of edp_set_batch_split run one after the other on
+ * launches of their own.  The rest of a wave of resident problems shares four
+ * launches: one zeroes the control words, one builds every cost volume, ONE
+ * persistent launch runs every scan pass of every problem (work items (pass,
+ * problem, row band) taken in order from a global queue, with bounded waits
+ * on the previous band and the previous pass of the same problem), and one
+ * evaluates every energy.  One status word covers the call.  Results are
+ * identical to solving each problem alone.  `probs` is host memory and is read during the
  * call only.  The call enqueues work and returns; it can be captured in a
- * CUDA graph (after one uncaptured call has set the kernels' attributes).
- * Problems at or above the size set by edp_set_batch_split run with launches
- * of their own inside the call. */
+ * CUDA graph (after one uncaptured call has set the kernels' attributes). */
 int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes, edp_stream_t stream);
 
 /* Split of edp_solve_batched (process-wide): a problem of at least
@@ -495,7 +507,8 @@ int edp_solve_batched(const edp_problem *probs, int n, void *ws, size_t ws_bytes
 int edp_set_batch_split(long long min_pixels);
 
 /* Reads the device status word of a workspace used by edp_solve /
- * edp_solve_images / edp_scanline_dp.  Synchronises `stream`. */
+ * edp_solve_weighted / edp_solve_images / edp_solve_windowed /
+ * edp_solve_batched / edp_scanline_dp.  Synchronises `stream`. */
 int edp_get_device_status(const void *ws, size_t ws_bytes, int *status, edp_stream_t stream);
 
 

@@ -495,7 +495,8 @@ bool plan_line2(const int32_t *C, int *const M[4], int W, int H, const Geometry 
 // One label axis in the same frame, four rows per block (a compute and four copy
 // warps each): a row below costs 0.5 us inside a block and 1.0 us between blocks,
 // a column 0.59 us against 0.55 us with one row per block (64 labels; 450x375:
-// 1.87 ms with four, 1.97 with three, 2.20 with two, 2.66 with one).
+// 1.87 ms with four, 1.97 with three, 2.20 with two, 2.66 with one, all with rings
+// of 8 columns; 1.85 with four and a row of records).
 bool plan_axis1(const int32_t *C, int *const M[4], int W, int H, const Geometry &g, const edp_params *p,
                 int32_t *labels, unsigned char *ws, SolvePlan *P) {
     if ((long long)p->lambda * 255 > pass_line2_max_lambda() || (reinterpret_cast<uintptr_t>(C) & 15)) return false;

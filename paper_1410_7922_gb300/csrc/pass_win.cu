@@ -1,7 +1,7 @@
 // pass_win.cu -- the cost of per-pixel label boxes for the windowed form of
 // EDP (used after a proposal): Eq. Cost_value restricted to each pixel's
-// n^R box.  The windowed scan pass is the WIN form of the band body in
-// pass_team.cuh.
+// n^R box.  The scan passes are in pass_win.cuh (two axes, linear prior) and in
+// the WIN form of the band body in pass_team.cuh (the rest).
 #include "common.cuh"
 #include "kernels.h"
 
