@@ -203,7 +203,8 @@ def set_tuning(rows_per_block: int = 0, labels_per_lane: int = 0, general_kernel
     multi-axis spaces its lane-group form, 3 = multi-axis spaces take the
     multi-axis kernel instead of the split line kernel, 4 = two-axis spaces
     take the line kernel with one label line per lane wherever it is built
-    (65 x 65 labels the split one), 5 = as 4, also at 65 x 65."""
+    (65 x 65 labels the split one), 5 = as 4, also at 65 x 65.  Pinned rows are
+    an upper bound; pinned warps go to a kernel that can run them."""
     _check(load().edp_set_tuning(int(rows_per_block), int(labels_per_lane), int(warps_per_row),
                                  int(general_kernel)), "set_tuning")
 
@@ -216,7 +217,7 @@ PAIRS_OFF, PAIRS_ON, PAIRS_AUTO = 0, 1, 2
 
 def set_pass_pairs(mode) -> None:
     """Pass schedule: PAIRS_OFF (one launch per pass), PAIRS_ON (paired sweeps
-    P1 + P2, P3 + P4) or PAIRS_AUTO (paired when every row band is resident;
+    P1 + P2, P3 + P4) or PAIRS_AUTO (paired where it is faster: see edp.h;
     the default).  A bool selects PAIRS_ON / PAIRS_OFF."""
     if isinstance(mode, bool):
         mode = PAIRS_ON if mode else PAIRS_OFF
@@ -572,8 +573,8 @@ NET_CHANNELS = (5, 32, 32, 32, 32, 32, 2)
 
 def set_fused_cost(on: bool) -> None:
     """edp_set_fused_cost: edp_solve_images computes the pair cost from the
-    images inside the split line kernel (True) or always builds the cost
-    volume first (False, the default)."""
+    images inside the split line kernel where that has a build for it (True,
+    65 x 65 labels) or always builds the cost volume first (False, the default)."""
     _check(load().edp_set_fused_cost(1 if on else 0), "set_fused_cost")
 
 
